@@ -65,9 +65,10 @@ typedef struct gm_config {
   uint64_t seed;       /* Philox key: initial picks (compress) / sampler (reconstruct) */
   double L;            /* periodic domain length; dx = L / C */
   double q;            /* species charge q_p; nonzero for the reconstructions (GM_ERR_ARG) */
-  int32_t threads_per_cell; /* EM CTA size: 0 = library choice, else 64, 128 or 256 */
-  int32_t smem_particles;   /* EM shared-memory tile in particles: 0 = library choice;
-                               cells with more particles use an L2-resident global tile */
+  int32_t threads_per_cell; /* EM lanes a cell's sums are split over (their order): 0 =
+                               library choice, else 64, 128 or 256 */
+  int32_t smem_particles;   /* EM shared-memory tile, at most, in particles: 0 = library
+                               choice; larger cells use an L2-resident global tile */
   int32_t precision;        /* penalised sweeps' M-step: 0 (default) = FP64 -- the
                                cross-warp statistic sums, covariance, its factor and
                                inverse, the weight -- with the convergence test's

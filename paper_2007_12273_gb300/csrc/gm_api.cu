@@ -10,11 +10,6 @@
 #include "gm_kernels.cuh"
 #include "std_kernel.cuh"
 
-namespace gmcr {
-int em_blocks_per_sm_d1(int nt, int fp64_mstep, int v_f64, size_t smem);
-int em_blocks_per_sm_d3(int nt, int fp64_mstep, int v_f64, size_t smem);
-}  // namespace gmcr
-
 namespace {
 
 thread_local std::string g_err;
@@ -266,11 +261,11 @@ static int compress_impl(const gm_config* cfg, int64_t C, int64_t n_particles,
   int nt = cfg->threads_per_cell > 0 ? cfg->threads_per_cell : 256;
   if (nt != 64 && nt != 128 && nt != 256)
     return fail(GM_ERR_ARG, "threads_per_cell must be 64, 128 or 256");
-  int cap = cfg->smem_particles > 0 ? cfg->smem_particles : (D == 1 ? 2560 : 3072);
-  cap &= ~3;  // pair records of 16 bytes behind D arrays of cap floats
+  // a shared tile takes up to 200 KB; by default any cell that fits may have one
+  const int most = 200 * 1024 / ((D + 4) * (int)sizeof(float));
+  int cap = cfg->smem_particles > 0 ? cfg->smem_particles & ~3 : most & ~3;
   if (cap < 4) cap = 4;
-  const size_t smem = (size_t)cap * (D + 4) * sizeof(float);
-  if (smem > 200 * 1024) return fail(GM_ERR_ARG, "smem_particles too large (%d)", cap);
+  if (cap > most) return fail(GM_ERR_ARG, "smem_particles too large (%d)", cap);
   if (cfg->precision != 0 && cfg->precision != 1)
     return fail(GM_ERR_ARG, "precision must be 0 (FP64 M-step) or 1 (FP32) (got %d)", cfg->precision);
   const int fp64_mstep = cfg->precision == 0;
@@ -321,13 +316,10 @@ static int compress_impl(const gm_config* cfg, int64_t C, int64_t n_particles,
   p.Kmax = cfg->Kmax;
   p.max_sweeps = cfg->max_sweeps;
   p.cap = cap;
+  p.v_f64 = v_is_f64 ? 1 : 0;
+  p.nvw = nt / 32;
   p.tol = cfg->tol;
   p.seed = cfg->seed;
-  const int per_sm = D == 1 ? gmcr::em_blocks_per_sm_d1(nt, fp64_mstep, v_is_f64, smem)
-                            : gmcr::em_blocks_per_sm_d3(nt, fp64_mstep, v_is_f64, smem);
-  if (per_sm < 1) return fail(GM_ERR_CUDA, "EM kernel does not fit on an SM (smem %zu)", smem);
-  int64_t grid = (int64_t)per_sm * sms;
-  if (grid > C) grid = C;
   if (init_K) {
     // supplied starts: the closed-form cells (one valid component, empty,
     // degenerate) one warp each; the EM kernel takes the list of the rest
@@ -358,8 +350,7 @@ static int compress_impl(const gm_config* cfg, int64_t C, int64_t n_particles,
     e = gmcr::launch_em_k1(D, v_is_f64, kp, sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "closed-form pre-pass launch");
   }
-  e = D == 1 ? gmcr::launch_em1(p, nt, fp64_mstep, v_is_f64, smem, (int)grid, s)
-             : gmcr::launch_em3(p, nt, fp64_mstep, v_is_f64, smem, (int)grid, s);
+  e = gmcr::launch_em(D, fp64_mstep, p, sms, s);
   if (e != cudaSuccess) return cuda_fail(e, "EM kernel launch");
   gmcr::trace_mark("em_kernel", s);
   if (x && init_K) {  // the records came from em_k1_kernel

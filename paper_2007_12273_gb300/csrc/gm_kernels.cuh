@@ -8,15 +8,11 @@
 
 namespace gmcr {
 
-// EM (compression); returns the launch error
-cudaError_t launch_em1(const EmParams& p, int nt, int fp64_mstep, int v_f64, size_t smem, int grid,
-                       cudaStream_t s);
+// EM (compression): p's work and limits set (all but team and granules);
+// returns the launch error
+cudaError_t launch_em(int D, int fp64_mstep, EmParams p, int sms, cudaStream_t s);
 size_t em_k1_raw_bytes(int D, int64_t C);
 cudaError_t launch_em_k1(int D, int v_f64, const K1Params& p, int sms, cudaStream_t s);
-cudaError_t launch_em3(const EmParams& p, int nt, int fp64_mstep, int v_f64, size_t smem, int grid,
-                       cudaStream_t s);
-// CTAs of an EM kernel that fit on one SM with `smem` dynamic bytes
-int em_blocks_per_sm(int D, int nt, int fp64_mstep, int v_f64, size_t smem);
 
 size_t deposit_ws_bytes(int64_t C);
 // rho from records that em_k1_kernel wrote (the deposit fused with the
