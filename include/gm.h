@@ -198,7 +198,8 @@ int gm_deposit_2d(const gm_config* cfg, const gm_mesh2d* mesh, const int64_t* ce
  * In: as gm_reconstruct with rho_target [Cy][Cx] and out_off [Cx Cy + 1]
  * (cfg->q must be nonzero).  Out: x_out, y_out [n_out] f64, v_out
  * [D][n_out] f64, alpha_out [n_out] f64, status_out [Cx Cy] uint32, dA_out
- * [Cx Cy] f64 (may be NULL).  Errors as gm_reconstruct (and a bad mesh);
+ * [Cx Cy] f64 (may be NULL); the particle arrays hold the draws until the
+ * call completes, as in gm_reconstruct.  Errors as gm_reconstruct (and a bad mesh);
  * a solve that stops at its iteration cap sets GM_ST_MM_NOT_CONVERGED.
  */
 int gm_reconstruct_2d(const gm_config* cfg, const gm_mesh2d* mesh, const int32_t* K,

@@ -556,7 +556,7 @@ int gm_reconstruct_2d(const gm_config* cfg, const gm_mesh2d* mesh, const int32_t
     return fail(GM_ERR_ARG, "an output particle pointer is NULL");
   if ((rc = check_device(nullptr))) return rc;
   void* ws = nullptr;
-  if ((rc = ws_get(gmcr::reconstruct2d_ws_bytes(cfg->D, mesh->Cx, mesh->Cy), &ws))) return rc;
+  if ((rc = ws_get(gmcr::reconstruct2d_ws_bytes(cfg->D, mesh->Cx, mesh->Cy, cfg->Kmax), &ws))) return rc;
   cudaError_t e = gmcr::launch_reconstruct2d(
       cfg->D, mesh->Cx, mesh->Cy, cfg->Kmax, K, params, W, rho_target, n_out, out_off, cfg->seed,
       mesh->Lx / (double)mesh->Cx, mesh->Ly / (double)mesh->Cy, cfg->q, cfg->shape_order, x_out,

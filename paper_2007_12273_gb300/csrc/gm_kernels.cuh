@@ -63,7 +63,7 @@ constexpr double kMesh2dTol = 1e-14;  // max |residual| / max |dx dy rho'| to st
 cudaError_t launch_deposit2d(int64_t Cx, int64_t Cy, const int64_t* cell_off, const double* x,
                              const double* y, const double* alpha, double dx, double dy, double q,
                              int order, double* part, double* rho, cudaStream_t s);
-size_t reconstruct2d_ws_bytes(int D, int64_t Cx, int64_t Cy);
+size_t reconstruct2d_ws_bytes(int D, int64_t Cx, int64_t Cy, int Kmax);
 cudaError_t launch_reconstruct2d(int D, int64_t Cx, int64_t Cy, int Kmax, const int32_t* K,
                                  const double* prm, const double* W, const double* rho_target,
                                  int64_t n_out, const int64_t* out_off, uint64_t seed, double dx,

@@ -23,85 +23,22 @@
 
 namespace gmcr {
 
-// Per-cell sums of the resampled particles, written by pass 1 (raw_words
-// doubles per cell).  A one-component cell with at most kFixMaxN particles
-// keeps exact 128-bit integer sums (see below), every other cell FP64 sums:
-//   integer: words (2t, 2t+1) hold sum t as (low, high) 64-bit halves, t =
-//            0, 1 the position sums, 2 .. 1+D the sums of f_d, 2+D .. 1+2D
-//            those of f_d^2;
-//   FP64:    words 0, 1 the position sums, 2 .. 1+D the sums of f_d (one
-//            component) or w_d (otherwise), 2+D the sum of |f|^2 or |w|^2.
-// The position sums are S1 = sum s, S2 = sum s^2 (quadratic B-spline) or
-// sum max(-s, 0), sum max(s, 0) (CIC), s = xi - 1/2 the particle's offset
-// from the cell centre; w = v - u = dz + f with f = L_z xi.
-template <int D>
-__host__ __device__ constexpr int raw_words() { return 2 * (2 + 2 * D); }
-__device__ __forceinline__ bool fixed_sums(int Kj, int64_t n) { return Kj == 1 && n <= kFixMaxN; }
-__device__ __forceinline__ __int128 load_i128(const double* p) {
-  const longlong2 v = *reinterpret_cast<const longlong2*>(p);
-  return ((__int128)v.y << 64) | (__int128)(unsigned long long)v.x;
-}
-// the exponents eq_d of the fixed-point f_d: |f_d| <= 9 sum_e |L_de|
-// (|xi| <= sqrt(-2 ln 2^-53) = 8.6) keeps f_d / 2^eq_d below 2^kFixBits
-template <int D>
-__device__ __forceinline__ void fix_exponents(const float* L, int (&eq)[D]) {
-  float bnd[D];
-  if (D == 1) {
-    bnd[0] = fabsf(L[0]);
-  } else {
-    bnd[0] = fabsf(L[0]);
-    bnd[1] = fabsf(L[1]) + fabsf(L[2]);
-    bnd[D - 1] = fabsf(L[3]) + fabsf(L[4]) + fabsf(L[5]);
-  }
-#pragma unroll
-  for (int d = 0; d < D; ++d) {
-    const int eb = (int)((__float_as_uint(9.0f * bnd[d]) >> 23) & 0xFFu);
-    eq[d] = (eb ? eb - 127 : -126) + 1 - kFixBits;
-  }
-}
-// Pass 1 stages each particle's draw in the caller's output slots of that
-// same particle, and pass 2 reads it back before it overwrites them with
-// the final values (one thread reads, then writes, each particle's slots,
-// so no other particle's staging is ever touched): x_out[p] holds the
-// position integer m0 (52 bits) and the component z (bits 56-63),
-// alpha_out[p] the FP32 pair (f_0, f_1), v_out[0][p] (D = 3) the FP32 f_2.
-// The second pass then needs neither the Philox draws nor the Box-Muller
-// transform of the first.
-template <int D>
-__device__ __forceinline__ void stage_draw(double* x_out, double* v_out, double* alpha_out,
-                                           int64_t p, uint64_t m0, int z, const float (&f)[D]) {
-  reinterpret_cast<unsigned long long*>(x_out)[p] = m0 | ((unsigned long long)(z & 0xFF) << 56);
-  reinterpret_cast<float2*>(alpha_out)[p] = make_float2(f[0], D == 3 ? f[1] : 0.0f);
-  if (D == 3) reinterpret_cast<float2*>(v_out)[p] = make_float2(f[D - 1], 0.0f);
-}
-template <int D>
-__device__ __forceinline__ void load_draw(const double* x_out, const double* v_out,
-                                          const double* alpha_out, int64_t p, uint64_t& m0, int& z,
-                                          float (&f)[D]) {
-  const unsigned long long t = reinterpret_cast<const unsigned long long*>(x_out)[p];
-  m0 = t & ((1ull << 52) - 1ull);
-  z = (int)(t >> 56);
-  const float2 a = reinterpret_cast<const float2*>(alpha_out)[p];
-  f[0] = a.x;
-  if (D == 3) {
-    f[1] = a.y;
-    f[D - 1] = reinterpret_cast<const float2*>(v_out)[p].x;
-  }
-}
-
+// Position sums of the 1D mesh: S1 = sum s, S2 = sum s^2 (quadratic B-spline)
+// or sum max(-s, 0), sum max(s, 0) (CIC), s = xi - 1/2 the particle's offset
+// from the cell centre.
 // the unit-weight shape sums of a cell's n particles on nodes j-1, j, j+1
 // (cs[0], cs[1], cs[2]): c- = (n/4 - S1 + S2) / 2, c+ = (n/4 + S1 + S2) / 2,
 // c0 = 3n/4 - S2 for the quadratic B-spline; c- = sum max(-s, 0),
 // c+ = sum max(s, 0), c0 = n - c- - c+ for CIC
-__device__ __forceinline__ void shape_sums(const double* rw, bool fixed, int order, int64_t n,
-                                           double (&cs)[3]) {
+template <int D>
+__device__ __forceinline__ void shape_sums(const RecRaw<D, 2>& r, int order, int64_t n, double (&cs)[3]) {
   double a0, a1;
-  if (fixed) {
-    a0 = i128_to_f64(load_i128(rw), -53);
-    a1 = i128_to_f64(load_i128(rw + 2), order == 1 ? -53 : -106);
+  if (r.fixed) {
+    a0 = i128_to_f64(load_i128(&r.w[0]), -53);
+    a1 = i128_to_f64(load_i128(&r.w[2]), order == 1 ? -53 : -106);
   } else {
-    a0 = rw[0];
-    a1 = rw[1];
+    a0 = r.w[0];
+    a1 = r.w[1];
   }
   const double nd = (double)n;
   if (order == 1) {
@@ -114,62 +51,67 @@ __device__ __forceinline__ void shape_sums(const double* rw, bool fixed, int ord
     cs[1] = 0.75 * nd - a1;
   }
 }
-// sum w (sw[0 .. D-1]) and sum |w|^2 (sw[D]) of a cell; for one component
-// w = dz + f with one dz, so sum w = n dz + sum f and
-// sum |w|^2 = n |dz|^2 + 2 dz . sum f + sum |f|^2
-template <int D>
-__device__ __forceinline__ void velocity_sums(const double* rw, bool fixed, int Kj,
-                                              const RecComp<D>& c0, int64_t n, double (&sw)[D + 1]) {
-  if (fixed) {
-    int eq[D];
-    fix_exponents<D>(c0.Lf, eq);
-    sw[D] = 0.0;
+// All sums of a cell on the integer pipe: the in-cell position offset
+// s = k 2^-53 with the odd integer k = 2 m0 - 2^52 + 1, and f_d (w_d) taken as
+// an integer multiple of 2^eq_d (exact within 2^-30 of the bound, to 2^-55
+// of it below).  A lane's 512 terms of k (|k| < 2^52) and of f_d / 2^eq_d fit
+// in 64 bits; the squares take 128.
+template <int D, bool kSeveral>
+__device__ __forceinline__ void sum_fixed(const RecCell<D>& rc, const long long (*dzq)[D], int64_t j, int64_t o,
+                                          int64_t n, uint64_t seed, int order, const int (&eq)[D], int lane,
+                                          double* x_out, double* v_out, double* alpha_out, RecRaw<D, 2>& rw) {
+  constexpr int NS = 2 + 2 * D;
+  __int128 sm[NS];
+  long long s0 = 0, sf[D];
+#pragma unroll
+  for (int t = 0; t < NS; ++t) sm[t] = 0;
+#pragma unroll
+  for (int d = 0; d < D; ++d) sf[d] = 0;
+  for (int64_t i = lane; i < n; i += 32) {
+    uint64_t m0;
+    int z;
+    float f[D];
+    sample_f<D>(rc, j, i, seed, m0, z, f);
+    stage_draw<D>(x_out, v_out, alpha_out, o + i, m0, z, f);
+    const long long k = 2ll * (long long)m0 - (1ll << 52) + 1ll;
+    if (order == 1) {
+      s0 += k < 0 ? -k : 0;
+      sm[1] += (__int128)(k > 0 ? k : 0);
+    } else {
+      s0 += k;
+      sm[1] += (__int128)k * (__int128)k;
+    }
 #pragma unroll
     for (int d = 0; d < D; ++d) {
-      sw[d] = i128_to_f64(load_i128(rw + 4 + 2 * d), eq[d]);
-      sw[D] += i128_to_f64(load_i128(rw + 4 + 2 * (D + d)), 2 * eq[d]);
+      long long fq = fixq(f[d], eq[d]);
+      if (kSeveral) fq += dzq[z][d];
+      sf[d] += fq;
+      sm[2 + D + d] += (__int128)fq * (__int128)fq;
     }
-  } else {
-#pragma unroll
-    for (int t = 0; t <= D; ++t) sw[t] = rw[2 + t];
   }
-  if (Kj == 1) {
-    const double nd = (double)n;
-    double dzf = 0.0, dz2 = 0.0;
+  sm[0] = (__int128)s0;
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-      const double dz = c0.dz[d];
-      dzf = fma(dz, sw[d], dzf);
-      dz2 = fma(dz, dz, dz2);
-      sw[d] = fma(nd, dz, sw[d]);
-    }
-    sw[D] = fma(nd, dz2, fma(2.0, dzf, sw[D]));
-  }
-}
-
-// Pass 0, one thread per cell: each cell's mixture data for the two particle
-// passes (prep_cell).
-template <int D>
-__global__ void recon_prep_kernel(int64_t C, int Kmax, const int32_t* K, const double* prm,
-                                  RecHead<D>* head, RecComp<D>* comp) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < C;
-       j += (int64_t)gridDim.x * blockDim.x)
-    prep_cell<D>(j, Kmax, K, prm, head, comp);
+  for (int d = 0; d < D; ++d) sm[2 + d] = (__int128)sf[d];
+  put_fixed<D, 2>(rw, sm, eq, lane);
 }
 
 // Pass 1, one warp per cell: the position and velocity sums of the cell's
-// resampled particles (raw_words layout above).
+// resampled particles (RecRaw).  Instruction issue bounds it: about 550 a
+// particle, two thirds of them the Philox blocks and the Box-Muller
+// transform.  Cells of several components take the integer sums too, with
+// w in the place of f: 18.8 M particles of 1-4 component 3V cells 0.50 -> 0.48
+// ms, 8.2 M of 1-8 component 1V cells 0.17 -> 0.13.
 template <int D, int NW>
 __global__ void __launch_bounds__(NW * 32, 6) recon_stats_kernel(int64_t C, int Kmax,
                                                               const RecHead<D>* head,
                                                               const RecComp<D>* comp,
                                                               const int64_t* out_off, int64_t n_out,
-                                                              uint64_t seed, int order, double* raw,
-                                                              double* x_out, double* v_out,
-                                                              double* alpha_out) {
+                                                              uint64_t seed, int order,
+                                                              RecRaw<D, 2>* raw, double* x_out,
+                                                              double* v_out, double* alpha_out) {
   constexpr int NA = 2 + D + 1;
-  constexpr int NS = 2 + 2 * D;
   __shared__ RecCell<D> rcs[NW];
+  __shared__ long long dzqs[NW][kMaxK][D];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   RecCell<D>& rc = rcs[wid];
   for (int64_t j = (int64_t)blockIdx.x * NW + wid; j < C; j += (int64_t)gridDim.x * NW) {
@@ -177,58 +119,13 @@ __global__ void __launch_bounds__(NW * 32, 6) recon_stats_kernel(int64_t C, int 
     __syncwarp();
     int64_t o, n;
     out_range(out_off, j, n_out, o, n);
-    double* rw = raw + (size_t)j * raw_words<D>();
-    if (fixed_sums(rc.K, n)) {
-      // one component: all sums on the integer pipe, exactly: the in-cell
-      // position offset s = k 2^-53 with the odd integer
-      // k = 2 m0 - 2^52 + 1, and f_d taken as an integer multiple of 2^eq_d
-      // (exact within 2^-30 of the bound, to 2^-55 of it below)
-      int eq[D];
-      fix_exponents<D>(rc.Lf[0], eq);
-      // a lane sums at most kFixMaxN / 32 = 512 terms, so its sums of
-      // k (|k| < 2^52) and of f_d / 2^eq_d (below 0.96 x 2^54: |xi| <= 8.6
-      // against the bound's 9) stay below 2^63 and fit in 64 bits; the
-      // squares take 128
-      __int128 sm[NS];
-      long long s0 = 0, sf[D];
-#pragma unroll
-      for (int t = 0; t < NS; ++t) sm[t] = 0;
-#pragma unroll
-      for (int d = 0; d < D; ++d) sf[d] = 0;
-      for (int64_t i = lane; i < n; i += 32) {
-        uint64_t m0;
-        int z;
-        float f[D];
-        sample_f<D>(rc, j, i, seed, m0, z, f);
-        stage_draw<D>(x_out, v_out, alpha_out, o + i, m0, z, f);
-        const long long k = 2ll * (long long)m0 - (1ll << 52) + 1ll;
-        if (order == 1) {
-          s0 += k < 0 ? -k : 0;
-          sm[1] += (__int128)(k > 0 ? k : 0);
-        } else {
-          s0 += k;
-          sm[1] += (__int128)k * (__int128)k;
-        }
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-          const long long fq = fixq(f[d], eq[d]);
-          sf[d] += fq;
-          sm[2 + D + d] += (__int128)fq * (__int128)fq;
-        }
-      }
-      sm[0] = (__int128)s0;
-#pragma unroll
-      for (int d = 0; d < D; ++d) sm[2 + d] = (__int128)sf[d];
-      __int128 mine = 0;
-#pragma unroll
-      for (int t = 0; t < NS; ++t) {
-#pragma unroll
-        for (int o2 = 16; o2 > 0; o2 >>= 1) sm[t] += shfl_xor_i128(sm[t], o2);
-        if (lane == t) mine = sm[t];
-      }
-      if (lane < NS)
-        *reinterpret_cast<longlong2*>(rw + 2 * lane) =
-            make_longlong2((long long)(unsigned long long)mine, (long long)(mine >> 64));
+    RecRaw<D, 2>& rw = raw[j];
+    int eq[D];
+    if (fix_plan<D>(rc, n, lane, eq, dzqs[wid])) {
+      // one component: w = f + dz is not formed (a loop of its own: with the
+      // several components' addition in it the 1.5e8-particle pass was 6 % slower)
+      if (rc.K == 1) sum_fixed<D, false>(rc, nullptr, j, o, n, seed, order, eq, lane, x_out, v_out, alpha_out, rw);
+      else sum_fixed<D, true>(rc, dzqs[wid], j, o, n, seed, order, eq, lane, x_out, v_out, alpha_out, rw);
     } else {
       double acc[NA];
 #pragma unroll
@@ -263,8 +160,10 @@ __global__ void __launch_bounds__(NW * 32, 6) recon_stats_kernel(int64_t C, int 
       }
 #pragma unroll
       for (int t = 0; t < NA; ++t) acc[t] = warp_sum(acc[t]);
-      if (lane == 0)
-        for (int t = 0; t < NA; ++t) rw[t] = acc[t];
+      if (lane == 0) {
+        for (int t = 0; t < NA; ++t) rw.w[t] = acc[t];
+        rw.fixed = 0;
+      }
     }
     __syncwarp();
   }
@@ -274,11 +173,9 @@ __global__ void __launch_bounds__(NW * 32, 6) recon_stats_kernel(int64_t C, int 
 // dA_{i+1}; M(i,j) = q * (shape sum of cell j's particles on node i).
 // rhs_i = dx (rho'_i - rho_i), rho_i dx = q sum_j alpha_j (shape sum).
 template <int D>
-__global__ void assemble_kernel(int64_t C, const RecHead<D>* head, const double* raw,
-                                const double* W, const int64_t* out_off, int64_t n_out,
+__global__ void assemble_kernel(int64_t C, const RecRaw<D, 2>* raw, const double* W, const int64_t* out_off, int64_t n_out,
                                 const double* rho_target, double dx, double q, int order, double* A,
                                 double* B, double* Cc, double* Dd) {
-  constexpr int RW = raw_words<D>();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < C;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t im = (i == 0) ? C - 1 : i - 1;
@@ -290,9 +187,9 @@ __global__ void assemble_kernel(int64_t C, const RecHead<D>* head, const double*
     const double a0 = n0 > 0 ? W[i] / (double)n0 : 0.0;
     const double ap = np > 0 ? W[ip] / (double)np : 0.0;
     double sm[3], s0[3], sp[3];
-    shape_sums(raw + (size_t)im * RW, fixed_sums(head[im].K, nm), order, nm, sm);
-    shape_sums(raw + (size_t)i * RW, fixed_sums(head[i].K, n0), order, n0, s0);
-    shape_sums(raw + (size_t)ip * RW, fixed_sums(head[ip].K, np), order, np, sp);
+    shape_sums<D>(raw[im], order, nm, sm);
+    shape_sums<D>(raw[i], order, n0, s0);
+    shape_sums<D>(raw[ip], order, np, sp);
     const double cm = sm[2];  // cell i-1 on node i
     const double c0 = s0[1];
     const double cp = sp[0];  // cell i+1 on node i
@@ -445,17 +342,10 @@ __global__ void mm_reconstruct_kernel(int64_t n, SolveWs ws, int P, double* x) {
 
 // After the mass-matrix solve, one thread per cell: the Lemons projection
 // coefficients (proj_coeffs) from the cell's velocity sums and dA, and the
-// cell's status.  For one component also cv = u + a (dz + beta), so that
-// the particle pass writes v = cv + a f.
-template <int D>
-struct RecCoef {
-  double a, beta[D], alpha_new, cv[D];
-  int skip;
-  int pad;
-};
+// cell's status.
 template <int D>
 __global__ void recon_coeffs_kernel(int64_t C, int Kmax, const RecHead<D>* head,
-                                    const RecComp<D>* comp, const double* raw,
+                                    const RecComp<D>* comp, const RecRaw<D, 2>* raw,
                                     const int64_t* out_off, int64_t n_out, const double* W,
                                     const double* dA, RecCoef<D>* coef, uint32_t* status_out) {
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < C;
@@ -465,92 +355,10 @@ __global__ void recon_coeffs_kernel(int64_t C, int Kmax, const RecHead<D>* head,
     const RecHead<D> h = head[j];
     const RecComp<D>& c0 = comp[(size_t)j * Kmax];
     double sw[D + 1];
-    velocity_sums<D>(raw + (size_t)j * raw_words<D>(), fixed_sums(h.K, n), h.K, c0, n, sw);
+    velocity_sums<D, 2>(raw[j], h.K, c0, n, sw);
     const ProjCoef<D> pc = proj_coeffs<D>(h.K, h.u, h.theta, n, W[j], dA[j], sw);
-    RecCoef<D> cf;
-    cf.a = pc.a;
-    cf.alpha_new = pc.alpha_new;
-    cf.skip = pc.skip;
-    cf.pad = 0;
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      cf.beta[d] = pc.beta[d];
-      // one component: v = u + a (dz + f + beta) = cv + a f (a = 1, beta = 0
-      // when skipped)
-      cf.cv[d] = h.K == 1 ? fma(pc.a, c0.dz[d] + pc.beta[d], h.u[d]) : 0.0;
-    }
-    coef[j] = cf;
+    coef[j] = make_coef<D>(pc, h, c0);
     status_out[j] = pc.status | (in_range ? 0u : GM_ST_BAD_RANGE);
-  }
-}
-
-// Pass 2, one warp per cell: the final particles (positions, projected
-// velocities, corrected weights) from the draws that pass 1 staged.
-template <int D, int NW>
-__global__ void __launch_bounds__(NW * 32) recon_emit_kernel(
-    int64_t C, int Kmax, const RecHead<D>* head, const RecComp<D>* comp, const RecCoef<D>* coef,
-    const int64_t* out_off, double dx, int64_t n_out, double* x_out, double* v_out,
-    double* alpha_out) {
-  __shared__ RecCell<D> rcs[NW];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  RecCell<D>& rc = rcs[wid];
-  for (int64_t j = (int64_t)blockIdx.x * NW + wid; j < C; j += (int64_t)gridDim.x * NW) {
-    load_prepped<D>(rc, j, Kmax, head, comp, lane);
-    const RecCoef<D> cf = coef[j];
-    __syncwarp();
-    int64_t o, n;
-    out_range(out_off, j, n_out, o, n);
-    const double aa = cf.a, an = cf.alpha_new;
-    if (rc.K == 1) {
-      // four particles per lane per step: their staged draws are all loaded
-      // before any of their slots is overwritten, so the loads of a step
-      // are in flight together
-      constexpr int U = 4;
-      int64_t i = lane;
-      for (; i + 32 * (U - 1) < n; i += 32 * U) {
-        uint64_t m0[U];
-        int z[U];
-        float f[U][D];
-#pragma unroll
-        for (int u = 0; u < U; ++u) load_draw<D>(x_out, v_out, alpha_out, o + i + 32 * u, m0[u], z[u], f[u]);
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int64_t p = o + i + 32 * u;
-          x_out[p] = __dmul_rn(cell_plus_u0((uint64_t)j, m0[u]), dx);
-          alpha_out[p] = an;
-#pragma unroll
-          for (int d = 0; d < D; ++d) v_out[(int64_t)d * n_out + p] = fma(aa, f2d_exact(f[u][d]), cf.cv[d]);
-        }
-      }
-      for (; i < n; i += 32) {
-        uint64_t m0;
-        int z;
-        float f[D];
-        load_draw<D>(x_out, v_out, alpha_out, o + i, m0, z, f);
-        x_out[o + i] = __dmul_rn(cell_plus_u0((uint64_t)j, m0), dx);
-        alpha_out[o + i] = an;
-#pragma unroll
-        for (int d = 0; d < D; ++d) v_out[(int64_t)d * n_out + o + i] = fma(aa, f2d_exact(f[d]), cf.cv[d]);
-      }
-    } else {
-      for (int64_t i = lane; i < n; i += 32) {
-        uint64_t m0;
-        int z;
-        float f[D];
-        double w[D];
-        load_draw<D>(x_out, v_out, alpha_out, o + i, m0, z, f);
-        draw_offset<D>(rc, z, f, w);
-        x_out[o + i] = __dmul_rn(cell_plus_u0((uint64_t)j, m0), dx);
-        alpha_out[o + i] = an;
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-          // v = u + w; projected: u + a (w + beta) (eqs. alpha, beta)
-          const double vp = cf.skip ? rc.u[d] + w[d] : fma(aa, w[d] + cf.beta[d], rc.u[d]);
-          v_out[(int64_t)d * n_out + o + i] = vp;
-        }
-      }
-    }
-    __syncwarp();
   }
 }
 
@@ -616,7 +424,7 @@ static size_t solve_doubles(const SolvePlan& pl) {
 // projection coefficients, then the FP64 arrays of the mass-matrix solve
 static size_t rec_bytes(int D, int64_t C, int Kmax, size_t* off_head, size_t* off_coef,
                         size_t* off_comp) {
-  const size_t raw = (size_t)C * (D == 1 ? raw_words<1>() : raw_words<3>()) * sizeof(double);
+  const size_t raw = (size_t)C * (D == 1 ? sizeof(RecRaw<1, 2>) : sizeof(RecRaw<3, 2>));
   const size_t hd = (size_t)C * (D == 1 ? sizeof(RecHead<1>) : sizeof(RecHead<3>));
   const size_t cf = (size_t)C * (D == 1 ? sizeof(RecCoef<1>) : sizeof(RecCoef<3>));
   const size_t cp = (size_t)C * Kmax * (D == 1 ? sizeof(RecComp<1>) : sizeof(RecComp<3>));
@@ -642,7 +450,7 @@ static void launch_passes(int64_t C, int Kmax, const int32_t* K, const double* p
                           const SolvePlan& pl, const SolveWs* lws, cudaStream_t s) {
   size_t oh, oc, op;
   rec_bytes(D, C, Kmax, &oh, &oc, &op);
-  double* raw = (double*)recs;
+  RecRaw<D, 2>* raw = (RecRaw<D, 2>*)recs;
   RecHead<D>* head = (RecHead<D>*)(recs + oh);
   RecCoef<D>* coef = (RecCoef<D>*)(recs + oc);
   RecComp<D>* comp = (RecComp<D>*)(recs + op);
@@ -657,7 +465,7 @@ static void launch_passes(int64_t C, int Kmax, const int32_t* K, const double* p
   recon_stats_kernel<D, NW><<<g, NW * 32, 0, s>>>(C, Kmax, head, comp, out_off, n_out, seed, order,
                                                   raw, x_out, v_out, alpha_out);
   trace_mark("recon_stats_kernel", s);
-  assemble_kernel<D><<<ga, 256, 0, s>>>(C, head, raw, W, out_off, n_out, rho_target, dx, q, order,
+  assemble_kernel<D><<<ga, 256, 0, s>>>(C, raw, W, out_off, n_out, rho_target, dx, q, order,
                                         A, B, Cc, Dd);
   trace_mark("assemble_kernel", s);
   {
@@ -682,8 +490,8 @@ static void launch_passes(int64_t C, int Kmax, const int32_t* K, const double* p
   recon_coeffs_kernel<D><<<ga, 256, 0, s>>>(C, Kmax, head, comp, raw, out_off, n_out, W, dA, coef,
                                             status_out);
   trace_mark("recon_coeffs_kernel", s);
-  recon_emit_kernel<D, NW><<<g, NW * 32, 0, s>>>(C, Kmax, head, comp, coef, out_off, dx, n_out,
-                                                 x_out, v_out, alpha_out);
+  recon_emit_kernel<D, NW, false><<<g, NW * 32, 0, s>>>(C, Kmax, head, comp, coef, out_off, C, dx, 0.0,
+                                                        n_out, x_out, nullptr, v_out, alpha_out);
   trace_mark("recon_emit_kernel", s);
 }
 

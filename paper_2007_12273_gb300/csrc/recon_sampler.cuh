@@ -46,10 +46,7 @@ struct RecCell {
   float Lf[kMaxK][NM];      // lower-triangular Cholesky factor (FP32), row-major
   double u[D];              // mixture mean sum_k w_k mu_k
   double theta;             // sum_k w_k (tr Sigma_k + |mu_k - u|^2)
-  double a, beta[D], alpha_new;
   int K;
-  int skip;
-  unsigned int status;
 };
 
 // FP32 lower-triangular Cholesky factor (row-major) of a component's
@@ -111,24 +108,7 @@ __device__ __forceinline__ void mix_head(const double* rj, int Kj, PutThr put_th
   theta = th;
 }
 
-// load cell j's mixture into the warp's RecCell: Cholesky factors on lanes
-// k < K, the rest on lane 0
-template <int D>
-__device__ void load_cell(RecCell<D>& rc, int64_t j, int Kmax, const int32_t* K,
-                          const double* prm, int lane) {
-  constexpr int P = 1 + D + D * (D + 1) / 2;
-  const int Kj = K[j];
-  const double* rj = prm + (size_t)j * Kmax * P;
-  if (lane < Kj) chol_f<D>(rj + (size_t)lane * P, rc.Lf[lane]);
-  if (lane == 0) {
-    rc.K = Kj;
-    mix_head<D>(
-        rj, Kj, [&](int q, long long t) { rc.thr[q] = t; },
-        [&](int q, int d, double x) { rc.dz[q][d] = x; }, rc.u, rc.theta);
-  }
-}
-
-// The same mixture data computed once per cell, by one thread per cell (the
+// A cell's mixture data computed once per cell, by one thread per cell (the
 // FP64 square roots and divisions then run 32 cells to a warp instruction),
 // and kept in the workspace for the two particle passes: per cell a head
 // (u, theta, K) and Kmax component records (threshold, dz, FP32 factor).
@@ -278,16 +258,6 @@ __device__ __forceinline__ void draw_offset(const RecCell<D>& rc, int z, const f
 #pragma unroll
   for (int d = 0; d < D; ++d) w[d] = rc.dz[z][d] + f2d_exact(f[d]);
 }
-// the same, drawing the particle
-template <int D>
-__device__ __forceinline__ void sample_particle(const RecCell<D>& rc, int64_t j, int64_t i,
-                                                uint64_t seed, uint64_t& m0, double (&w)[D]) {
-  int z;
-  float f[D];
-  sample_f<D>(rc, j, i, seed, m0, z, f);
-  draw_offset<D>(rc, z, f, w);
-}
-
 // the 52 leading bits of the y uniform of particle i of cell j on a 2D mesh
 // (Philox block 3, words 0-1)
 __device__ __forceinline__ uint64_t sample_y_bits(int64_t j, int64_t i, uint64_t seed) {
@@ -302,8 +272,6 @@ __device__ __forceinline__ double centred52(uint64_t m) {
   return m >= (1ull << 51) ? odd_2m53(2ull * m - (1ull << 52) + 1ull, false)
                            : odd_2m53((1ull << 52) - 2ull * m - 1ull, true);
 }
-// the position uniform u0 = (m + 1/2) 2^-52 = (2 m + 1) 2^-53 of a 52-bit m
-__device__ __forceinline__ double uniform_pos52(uint64_t m) { return odd_2m53(2ull * m + 1ull, false); }
 // j + u0 rounded to the nearest double (ties to even), as the FP64 addition
 // (double)j + u0 gives it, on the integer pipe, for 0 <= j < 2^52: with L
 // the leading bit of j the sum's 53-bit significand in units of 2^(L - 52)
@@ -367,17 +335,308 @@ __device__ __forceinline__ ProjCoef<D> proj_coeffs(int K, const double* u, doubl
   pc.status = st;
   return pc;
 }
-// the same on the warp's RecCell (lane 0); returns the status
+// ---------------------------------------------------------------------------
+// Pass 1's per-cell record and the staged draws (both meshes)
+// ---------------------------------------------------------------------------
+// Sums of a cell's resampled particles.  A cell with components and at most
+// kFixMaxN particles keeps integer sums (fixed = 1), every other cell FP64
+// sums:
+//   integer: sum t as (low, high) 64-bit halves in words (2t, 2t+1): first
+//            the NP position sums, then D sums of f_d (one component) or
+//            w_d (several) in units of 2^eq_d, then D sums of their squares;
+//   FP64:    words 0 .. NP-1 the position sums, then the D sums of f_d (one
+//            component) or w_d (otherwise) and the sum of |f|^2 or |w|^2.
+// w = v - u = dz + f with f = L_z xi.  An FP64 addition costs as much as some
+// sixty integer instructions here, and the integer sums carry no rounding
+// from particle to particle.
+template <int D, int NP>
+struct alignas(16) RecRaw {
+  static constexpr int NS = NP + 2 * D;
+  double w[2 * NS];
+  int eq[3];
+  int fixed;
+};
+__device__ __forceinline__ __int128 load_i128(const double* p) {
+  const longlong2 v = *reinterpret_cast<const longlong2*>(p);
+  return ((__int128)v.y << 64) | (__int128)(unsigned long long)v.x;
+}
+// bound of |f_d| by the factor's rows: |xi| <= sqrt(-2 ln 2^-53) = 8.6 < 9
 template <int D>
-__device__ unsigned int projection_coeffs(RecCell<D>& rc, int64_t n, double Wj, double dAj,
-                                          const double* sw) {
-  const ProjCoef<D> pc = proj_coeffs<D>(rc.K, rc.u, rc.theta, n, Wj, dAj, sw);
-  rc.alpha_new = pc.alpha_new;
-  rc.a = pc.a;
-  for (int d = 0; d < D; ++d) rc.beta[d] = pc.beta[d];
-  rc.skip = pc.skip;
-  rc.status = pc.status;
-  return pc.status;
+__device__ __forceinline__ void row_bounds(const float* L, float (&bnd)[D]) {
+  if (D == 1) {
+    bnd[0] = 9.0f * fabsf(L[0]);
+  } else {
+    bnd[0] = 9.0f * fabsf(L[0]);
+    bnd[1] = 9.0f * (fabsf(L[1]) + fabsf(L[2]));
+    bnd[D - 1] = 9.0f * (fabsf(L[3]) + fabsf(L[4]) + fabsf(L[5]));
+  }
+}
+// exponent eq with v / 2^eq below 2^bits for |v| <= b
+__device__ __forceinline__ int fix_exponent(float b, int bits) {
+  const int eb = (int)((__float_as_uint(b) >> 23) & 0xFFu);
+  return (eb ? eb - 127 : -126) + 1 - bits;
+}
+// d / 2^eq rounded to the nearest integer (ties away from zero), from the
+// bit pattern of an FP64 d with |d| < 2^(eq + 54)
+__device__ __forceinline__ long long fixq_d(double d, int eq) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+  const int e = (int)((u >> 52) & 0x7FFull);
+  const long long m = (long long)((u & ((1ull << 52) - 1ull)) | (e ? (1ull << 52) : 0ull));
+  const int sh = (e ? e : 1) - 1075 - eq;  // d = m 2^(e - 1075)
+  long long r = 0;
+  if (sh >= 0) r = m << (sh < 10 ? sh : 10);
+  else if (sh > -60) r = (m + (1ll << (-sh - 1))) >> (-sh);
+  return (u >> 63) ? -r : r;
+}
+// The fixed-point plan of a cell in the warp's RecCell: the exponents eq and
+// (several components) dzq[k] = dz_k / 2^eq.  One component: f alone, kFixBits
+// bits, so that a lane's kFixMaxN / 32 = 512 terms (0.96 x 2^54 each) stay
+// below 2^63; several: w, one bit less.  False (no component, too many
+// particles, or offsets beyond FP32) for the FP64 sums.
+template <int D>
+__device__ __forceinline__ bool fix_plan(const RecCell<D>& rc, int64_t n, int lane, int (&eq)[D],
+                                         long long (*dzq)[D]) {
+  const int K = rc.K;
+  if (K < 1 || n > kFixMaxN) return false;
+  float b[D];
+  row_bounds<D>(rc.Lf[lane < K ? lane : 0], b);
+  if (K == 1) {
+#pragma unroll
+    for (int d = 0; d < D; ++d) eq[d] = fix_exponent(b[d], kFixBits);
+    return true;
+  }
+  bool ok = true;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    b[d] = lane < K ? (fabsf((float)rc.dz[lane][d]) + b[d]) * 1.00001f : 0.0f;
+    b[d] = warp_max(b[d]);
+    ok = ok && b[d] < 1e38f;
+    eq[d] = fix_exponent(b[d], kFixBits - 1);
+  }
+  if (!__all_sync(0xffffffffu, ok)) return false;
+  if (lane < K)
+#pragma unroll
+    for (int d = 0; d < D; ++d) dzq[lane][d] = fixq_d(rc.dz[lane][d], eq[d]);
+  __syncwarp();
+  return true;
+}
+// the warp's integer sums sm into cell record r
+template <int D, int NP>
+__device__ __forceinline__ void put_fixed(RecRaw<D, NP>& r, __int128 (&sm)[NP + 2 * D], const int (&eq)[D],
+                                          int lane) {
+  __int128 mine = 0;
+#pragma unroll
+  for (int t = 0; t < NP + 2 * D; ++t) {
+#pragma unroll
+    for (int o2 = 16; o2 > 0; o2 >>= 1) sm[t] += shfl_xor_i128(sm[t], o2);
+    if (lane == t) mine = sm[t];
+  }
+  if (lane < NP + 2 * D)
+    *reinterpret_cast<longlong2*>(&r.w[2 * lane]) =
+        make_longlong2((long long)(unsigned long long)mine, (long long)(mine >> 64));
+  if (lane == 0) {
+#pragma unroll
+    for (int d = 0; d < D; ++d) r.eq[d] = eq[d];
+    r.fixed = 1;
+  }
+}
+// Pass 1 stages each particle's draw in the caller's output slots of that
+// same particle, and pass 2 reads it back before it overwrites them with
+// the final values (one thread reads, then writes, each particle's slots,
+// so no other particle's staging is ever touched): x_out[p] holds the
+// position integer m0 (52 bits) and the component z (bits 56-63),
+// alpha_out[p] the FP32 pair (f_0, f_1), v_out[0][p] (D = 3) the FP32 f_2.
+// The second pass then needs neither the Philox draws nor the Box-Muller
+// transform of the first.
+template <int D>
+__device__ __forceinline__ void stage_draw(double* x_out, double* v_out, double* alpha_out,
+                                           int64_t p, uint64_t m0, int z, const float (&f)[D]) {
+  reinterpret_cast<unsigned long long*>(x_out)[p] = m0 | ((unsigned long long)(z & 0xFF) << 56);
+  reinterpret_cast<float2*>(alpha_out)[p] = make_float2(f[0], D == 3 ? f[1] : 0.0f);
+  if (D == 3) reinterpret_cast<float2*>(v_out)[p] = make_float2(f[D - 1], 0.0f);
+}
+template <int D>
+__device__ __forceinline__ void load_draw(const double* x_out, const double* v_out,
+                                          const double* alpha_out, int64_t p, uint64_t& m0, int& z,
+                                          float (&f)[D]) {
+  const unsigned long long t = reinterpret_cast<const unsigned long long*>(x_out)[p];
+  m0 = t & ((1ull << 52) - 1ull);
+  z = (int)(t >> 56);
+  const float2 a = reinterpret_cast<const float2*>(alpha_out)[p];
+  f[0] = a.x;
+  if (D == 3) {
+    f[1] = a.y;
+    f[D - 1] = reinterpret_cast<const float2*>(v_out)[p].x;
+  }
+}
+
+// sum w (sw[0 .. D-1]) and sum |w|^2 (sw[D]) of a cell; for one component
+// w = dz + f with one dz, so sum w = n dz + sum f and
+// sum |w|^2 = n |dz|^2 + 2 dz . sum f + sum |f|^2
+template <int D, int NP>
+__device__ __forceinline__ void velocity_sums(const RecRaw<D, NP>& r, int Kj, const RecComp<D>& c0,
+                                              int64_t n, double (&sw)[D + 1]) {
+  if (r.fixed) {
+    sw[D] = 0.0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      sw[d] = i128_to_f64(load_i128(&r.w[2 * (NP + d)]), r.eq[d]);
+      sw[D] += i128_to_f64(load_i128(&r.w[2 * (NP + D + d)]), 2 * r.eq[d]);
+    }
+  } else {
+#pragma unroll
+    for (int t = 0; t <= D; ++t) sw[t] = r.w[NP + t];
+  }
+  if (Kj == 1) {
+    const double nd = (double)n;
+    double dzf = 0.0, dz2 = 0.0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const double dz = c0.dz[d];
+      dzf = fma(dz, sw[d], dzf);
+      dz2 = fma(dz, dz, dz2);
+      sw[d] = fma(nd, dz, sw[d]);
+    }
+    sw[D] = fma(nd, dz2, fma(2.0, dzf, sw[D]));
+  }
+}
+
+// Pass 0, one thread per cell: each cell's mixture data for the two particle
+// passes (prep_cell).
+template <int D>
+__global__ void recon_prep_kernel(int64_t C, int Kmax, const int32_t* K, const double* prm,
+                                  RecHead<D>* head, RecComp<D>* comp) {
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < C;
+       j += (int64_t)gridDim.x * blockDim.x)
+    prep_cell<D>(j, Kmax, K, prm, head, comp);
+}
+
+// a cell's projection for pass 2: the scale a and shift beta, the corrected
+// weight and, for one component, cv = u + a (dz + beta), so that the particle
+// pass writes v = cv + a f (a = 1 and beta = 0 when the projection is skipped)
+template <int D>
+struct RecCoef {
+  double a, beta[D], alpha_new, cv[D];
+};
+template <int D>
+__device__ __forceinline__ RecCoef<D> make_coef(const ProjCoef<D>& pc, const RecHead<D>& h,
+                                                const RecComp<D>& c0) {
+  RecCoef<D> cf;
+  cf.a = pc.a;
+  cf.alpha_new = pc.alpha_new;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    cf.beta[d] = pc.beta[d];
+    cf.cv[d] = h.K == 1 ? fma(pc.a, c0.dz[d] + pc.beta[d], h.u[d]) : 0.0;
+  }
+  return cf;
+}
+
+// Pass 2, one warp per cell: the final particles (positions, projected
+// velocities, corrected weights) from the draws that pass 1 staged (on the 2D
+// mesh y_out holds the y uniform's 52 bits).
+template <int D, int NW, bool kMesh2d>
+__global__ void __launch_bounds__(NW * 32) recon_emit_kernel(
+    int64_t C, int Kmax, const RecHead<D>* head, const RecComp<D>* comp, const RecCoef<D>* coef,
+    const int64_t* out_off, int64_t Cx, double dx, double dy, int64_t n_out, double* x_out, double* y_out,
+    double* v_out, double* alpha_out) {
+  __shared__ RecCell<D> rcs[NW];
+  __shared__ double cvs[NW][kMaxK][D];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  RecCell<D>& rc = rcs[wid];
+  for (int64_t j = (int64_t)blockIdx.x * NW + wid; j < C; j += (int64_t)gridDim.x * NW) {
+    load_prepped<D>(rc, j, Kmax, head, comp, lane);
+    const RecCoef<D> cf = coef[j];
+    __syncwarp();
+    int64_t o, n;
+    out_range(out_off, j, n_out, o, n);
+    const double aa = cf.a, an = cf.alpha_new;
+    const uint64_t jx = kMesh2d ? (uint64_t)(j % Cx) : (uint64_t)j, jy = kMesh2d ? (uint64_t)(j / Cx) : 0;
+    if (rc.K == 1) {
+      // four particles per lane per step: their staged draws are all loaded
+      // before any of their slots is overwritten, so the loads of a step
+      // are in flight together
+      constexpr int U = 4;
+      int64_t i = lane;
+      for (; i + 32 * (U - 1) < n; i += 32 * U) {
+        uint64_t m0[U], my[U];
+        int z[U];
+        float f[U][D];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          load_draw<D>(x_out, v_out, alpha_out, o + i + 32 * u, m0[u], z[u], f[u]);
+          my[u] = kMesh2d ? reinterpret_cast<const unsigned long long*>(y_out)[o + i + 32 * u] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t p = o + i + 32 * u;
+          x_out[p] = __dmul_rn(cell_plus_u0(jx, m0[u]), dx);
+          if (kMesh2d) y_out[p] = __dmul_rn(cell_plus_u0(jy, my[u]), dy);
+          alpha_out[p] = an;
+#pragma unroll
+          for (int d = 0; d < D; ++d) v_out[(int64_t)d * n_out + p] = fma(aa, f2d_exact(f[u][d]), cf.cv[d]);
+        }
+      }
+      for (; i < n; i += 32) {
+        uint64_t m0, my = 0;
+        int z;
+        float f[D];
+        load_draw<D>(x_out, v_out, alpha_out, o + i, m0, z, f);
+        if (kMesh2d) my = reinterpret_cast<const unsigned long long*>(y_out)[o + i];
+        x_out[o + i] = __dmul_rn(cell_plus_u0(jx, m0), dx);
+        if (kMesh2d) y_out[o + i] = __dmul_rn(cell_plus_u0(jy, my), dy);
+        alpha_out[o + i] = an;
+#pragma unroll
+        for (int d = 0; d < D; ++d) v_out[(int64_t)d * n_out + o + i] = fma(aa, f2d_exact(f[d]), cf.cv[d]);
+      }
+    } else {
+      // several components: v = c_z + a f with c_k = u + a (dz_k + beta) once
+      // per component (one FP64 operation per dimension instead of three:
+      // 0.47 -> 0.26 ms for 18.8 M particles in 3V, 0.12 -> 0.07 for 8.2 M in 1V); no component: v = 0
+      if (lane < rc.K)
+#pragma unroll
+        for (int d = 0; d < D; ++d) cvs[wid][lane][d] = fma(aa, rc.dz[lane][d] + cf.beta[d], rc.u[d]);
+      if (rc.K == 0 && lane < D) cvs[wid][0][lane] = 0.0;
+      __syncwarp();
+      const int zmax = rc.K > 0 ? rc.K - 1 : 0;
+      constexpr int U = 2;
+      int64_t i = lane;
+      for (; i + 32 * (U - 1) < n; i += 32 * U) {
+        uint64_t m0[U], my[U];
+        int z[U];
+        float f[U][D];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          load_draw<D>(x_out, v_out, alpha_out, o + i + 32 * u, m0[u], z[u], f[u]);
+          my[u] = kMesh2d ? reinterpret_cast<const unsigned long long*>(y_out)[o + i + 32 * u] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t p = o + i + 32 * u;
+          const double* cv = cvs[wid][z[u] < zmax ? z[u] : zmax];
+          x_out[p] = __dmul_rn(cell_plus_u0(jx, m0[u]), dx);
+          if (kMesh2d) y_out[p] = __dmul_rn(cell_plus_u0(jy, my[u]), dy);
+          alpha_out[p] = an;
+#pragma unroll
+          for (int d = 0; d < D; ++d) v_out[(int64_t)d * n_out + p] = fma(aa, f2d_exact(f[u][d]), cv[d]);
+        }
+      }
+      for (; i < n; i += 32) {
+        uint64_t m0, my = 0;
+        int z;
+        float f[D];
+        load_draw<D>(x_out, v_out, alpha_out, o + i, m0, z, f);
+        if (kMesh2d) my = reinterpret_cast<const unsigned long long*>(y_out)[o + i];
+        const double* cv = cvs[wid][z < zmax ? z : zmax];
+        x_out[o + i] = __dmul_rn(cell_plus_u0(jx, m0), dx);
+        if (kMesh2d) y_out[o + i] = __dmul_rn(cell_plus_u0(jy, my), dy);
+        alpha_out[o + i] = an;
+#pragma unroll
+        for (int d = 0; d < D; ++d) v_out[(int64_t)d * n_out + o + i] = fma(aa, f2d_exact(f[d]), cv[d]);
+      }
+    }
+    __syncwarp();
+  }
 }
 
 }  // namespace gmcr
