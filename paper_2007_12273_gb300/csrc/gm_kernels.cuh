@@ -71,12 +71,10 @@ cudaError_t launch_reconstruct2d(int D, int64_t Cx, int64_t Cy, int Kmax, const 
                                  double* v_out, double* alpha_out, uint32_t* status_out,
                                  double* dA_user, void* ws, cudaStream_t s);
 
-// BF16 tcgen05 GEMM: C = A B^T (+bias, ReLU, mask), see tc_gemm.cu
-size_t tc_gemm_smem(int bn);
-cudaError_t launch_tc_gemm(const void* A, const void* B, int M, int N, int K, int lda, int ldb,
-                           const float* bias, int relu, const void* mask, int ldm, float* Cf,
-                           void* Cb, int ldc, unsigned int* err, cudaStream_t s,
-                           int accumulate = 0);
+// BF16 tcgen05 GEMM: C = A B^T (+ A2 B^T) (+bias, ReLU, mask), see tc_gemm.cu
+cudaError_t launch_tc_gemm(const void* A, const void* A2, const void* B, int M, int N, int K, int lda,
+                           int ldb, const float* bias, int relu, const void* mask, int ldm, float* Cf,
+                           void* Cb, int ldc, unsigned int* err, cudaStream_t s);
 
 }  // namespace gmcr
 
@@ -90,16 +88,33 @@ cudaError_t launch_targets(int D, int64_t C, int Kmax, int O, const int32_t* K, 
 cudaError_t launch_decode(int D, int64_t C, int Kmax, int O, const float* out, const double* wstat,
                           const int64_t* cell_off, float presence_logit, int32_t* K0, double* prm,
                           cudaStream_t s);
+// a gradient's BF16 parts, row-major and transposed, and the gradient itself
+// (mlp_kernels.cu); rows a multiple of kGradRows
+constexpr int kGradRows = 64;
+struct GradOut {
+  void *hi, *lo, *hiT, *loT;  // [M][C] (may be NULL), [C][M]
+  float* g;                   // [M][C]
+};
+// of the loss with respect to the network's output (and the loss itself)
 cudaError_t launch_loss_grad(int B, int O, int D, int Kmax, const float* out, const float* T,
-                             const float* Mk, float* G32, void* G16, double* loss, cudaStream_t s);
-cudaError_t launch_transpose_bf16(int R, int Cc, const void* in, int ldi, void* out, int ldo,
-                                  cudaStream_t s);
-cudaError_t launch_colsum(int R, int Cc, const void* G, int ld, int g_is_bf16, float* db,
-                          cudaStream_t s);
-cudaError_t launch_adam(int n_out, int n_in, float* w, const float* g, float* m, float* v, float lr,
-                        int step, void* w16, void* wt16, cudaStream_t s);
+                             const float* Mk, const GradOut& g, double* loss, cudaStream_t s);
+// of a layer's pre-activations: g.g, set to 0 where its ReLU output is not > 0
+cudaError_t launch_grad_prep(int M, int Cc, const void* mask, const GradOut& g, cudaStream_t s);
+struct TransposeJobs {
+  const void* in[4];
+  void* out[4];
+  int cols[4];
+};
+cudaError_t launch_transposes(int M, const TransposeJobs& t, cudaStream_t s);
+// bias gradients (the column sums of G [M][rows]) and, if lr > 0, Adam on
+// every tensor with the BF16 copies and transposes of the weights
+struct UpdateJobs {
+  float *W[4], *b[4], *gW[4], *gb[4], *mW[4], *vW[4], *mb[4], *vb[4];
+  void *W16[4], *WT16[4];
+  const float* G[4];
+  int rows[4], cols[4], M;
+};
+cudaError_t launch_update(const UpdateJobs& u, float lr, int step, cudaStream_t s);
 cudaError_t launch_cast_weights(int n_out, int n_in, const float* w, void* w16, void* wt16,
                                 cudaStream_t s);
-cudaError_t launch_split_bf16(int64_t total, int cols, float* x, const void* mask, int ldm,
-                              void* hi, void* lo, cudaStream_t s);
 }  // namespace gmcr

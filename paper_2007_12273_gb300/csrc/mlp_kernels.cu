@@ -225,104 +225,171 @@ __global__ void targets_kernel(int64_t C, int Kmax, int O, const int32_t* K, con
 }
 
 // ---------------------------------------------------------------------------
-// loss and d loss / d out (mean over the batch of B rows)
+// the training step's passes between its GEMMs.  A batch's matrices are a
+// megabyte or less, so a pass costs its launch and its latency; each element
+// is read once and leaves in every form that the next GEMMs take.
 // ---------------------------------------------------------------------------
-__global__ void loss_grad_kernel(int B, int O, int SP, int nslot, const float* out, const float* T,
-                                 const float* Mk, float* G32, __nv_bfloat16* G16, double* loss) {
+constexpr int kGT = 32;  // a CTA's columns, and the side of its transposed tiles
+
+// kGradRows x kGT elements of a gradient by 32 x 8 threads: value(row, col)
+// stored as it is and as BF16 parts hi = bf16(v), lo = bf16(v - hi), these
+// row-major and transposed (through shared memory)
+template <class F>
+__device__ __forceinline__ void grad_tile(int M, int Cc, const GradOut& g, F value) {
+  __shared__ __nv_bfloat162 tile[kGT][kGT + 1];
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int c0 = blockIdx.x * kGT, r0 = blockIdx.y * kGradRows, col = c0 + tx;
+  __nv_bfloat16 *hi = (__nv_bfloat16*)g.hi, *lo = (__nv_bfloat16*)g.lo;
+  __nv_bfloat16 *hiT = (__nv_bfloat16*)g.hiT, *loT = (__nv_bfloat16*)g.loT;
+  for (int sub = 0; sub < kGradRows; sub += kGT) {
+#pragma unroll
+    for (int i = 0; i < kGT; i += 8) {
+      const int row = r0 + sub + ty + i;
+      const float v = col < Cc ? value(row, col) : 0.0f;
+      const __nv_bfloat16 h = __float2bfloat16(v), l = __float2bfloat16(v - __bfloat162float(h));
+      if (col < Cc) {
+        const size_t at = (size_t)row * Cc + col;
+        g.g[at] = v;
+        if (hi) {
+          hi[at] = h;
+          lo[at] = l;
+        }
+      }
+      tile[ty + i][tx] = __halves2bfloat162(h, l);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kGT; i += 8) {
+      const int cT = c0 + ty + i, rT = r0 + sub + tx;
+      if (cT < Cc) {
+        const __nv_bfloat162 t = tile[tx][ty + i];
+        hiT[(size_t)cT * M + rT] = __low2bfloat16(t);
+        loT[(size_t)cT * M + rT] = __high2bfloat16(t);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// loss and d loss / d out (mean over the batch of B rows)
+__global__ void __launch_bounds__(256) loss_grad_kernel(int B, int O, int SP, int nslot, const float* out,
+                                                        const float* T, const float* Mk, GradOut g,
+                                                        double* loss) {
   __shared__ double red[8];
   double acc = 0.0;
   const float inv = 1.0f / (float)B;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (int64_t)B * O;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int col = (int)(i % O);
+  grad_tile(B, O, g, [&](int row, int col) {
+    const size_t i = (size_t)row * O + col;
     const float p = out[i], t = T[i];
-    float g = 0.0f;
+    float gr = 0.0f;
     if (col < nslot * SP && col % SP == 0) {  // presence logit: BCE
       const float sp = p > 0.0f ? p + log1pf(expf(-p)) : log1pf(expf(p));
       acc += (double)(sp - t * p);
-      g = 1.0f / (1.0f + expf(-p)) - t;
+      gr = 1.0f / (1.0f + expf(-p)) - t;
     } else if (Mk[i] > 0.0f) {
       const float d = p - t;
       acc += (double)d * d;
-      g = 2.0f * d;
+      gr = 2.0f * d;
     }
-    g *= inv;
-    G32[i] = g;
-    G16[i] = __float2bfloat16(g);
-  }
+    return gr * inv;
+  });
   acc = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  if (threadIdx.x == 0) red[threadIdx.y] = acc;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
     double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
+    for (int w = 0; w < 8; ++w) s += red[w];
     atomicAdd(loss, s / (double)B);
   }
 }
 
-// out[c][r] = in[r][c] (BF16), 32 x 32 tiles
-__global__ void transpose_bf16_kernel(int R, int Cc, const __nv_bfloat16* in, int ldi,
-                                      __nv_bfloat16* out, int ldo) {
-  __shared__ __nv_bfloat16 tile[32][33];
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
+// g.g zeroed where the layer's output is not positive
+__global__ void __launch_bounds__(256) grad_prep_kernel(int M, int Cc, const __nv_bfloat16* mask, GradOut g) {
+  grad_tile(M, Cc, g, [&](int row, int col) {
+    const size_t i = (size_t)row * Cc + col;
+    return __bfloat162float(mask[i]) > 0.0f ? g.g[i] : 0.0f;
+  });
+}
+
+// out[c][r] = in[r][c] (BF16), 32 x 32 tiles, one matrix per blockIdx.z
+__global__ void __launch_bounds__(256) transposes_kernel(int M, TransposeJobs t) {
+  __shared__ __nv_bfloat16 tile[kGT][kGT + 1];
+  const int z = blockIdx.z, Cc = t.cols[z];
+  const int r0 = blockIdx.y * kGT, c0 = blockIdx.x * kGT;
+  if (c0 >= Cc) return;
+  const __nv_bfloat16* in = (const __nv_bfloat16*)t.in[z];
+  __nv_bfloat16* out = (__nv_bfloat16*)t.out[z];
+  for (int i = threadIdx.y; i < kGT; i += 8) {
     const int r = r0 + i, c = c0 + threadIdx.x;
-    tile[i][threadIdx.x] = (r < R && c < Cc) ? in[(size_t)r * ldi + c] : __float2bfloat16(0.0f);
+    tile[i][threadIdx.x] = (r < M && c < Cc) ? in[(size_t)r * Cc + c] : __float2bfloat16(0.0f);
   }
   __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
+  for (int i = threadIdx.y; i < kGT; i += 8) {
     const int c = c0 + i, r = r0 + threadIdx.x;
-    if (c < Cc && r < R) out[(size_t)c * ldo + r] = tile[threadIdx.x][i];
+    if (c < Cc && r < M) out[(size_t)c * M + r] = tile[threadIdx.x][i];
   }
 }
 
-// db[c] = sum_r G[r][c] (FP32 or BF16 input)
-template <typename TG>
-__global__ void colsum_kernel(int R, int Cc, const TG* G, int ld, float* db) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < Cc; c += gridDim.x * blockDim.x) {
-    float s = 0.0f;
-    for (int r = 0; r < R; ++r) s += (float)G[(size_t)r * ld + c];
-    db[c] = s;
-  }
+__device__ __forceinline__ float adam_step(float* w, float gi, float* m, float* v, int64_t i, float lr,
+                                           float b1, float b2, float eps, float c1, float c2) {
+  const float mi = b1 * m[i] + (1.0f - b1) * gi;
+  const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
+  m[i] = mi;
+  v[i] = vi;
+  const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  w[i] = wi;
+  return wi;
 }
 
-// Adam on one tensor [n_out][n_in] (n_in = 1 for a bias); refreshes the BF16
-// copy and its transpose when given
-__global__ void adam_kernel(int n_out, int n_in, float* w, const float* g, float* m, float* v,
-                            float lr, float b1, float b2, float eps, float c1, float c2,
-                            __nv_bfloat16* w16, __nv_bfloat16* wt16) {
+// blockIdx.y = layer.  The first kBiasCtas blocks of a layer sum kGT columns
+// of its gradient each: a column is added in row order by one thread (the
+// order is part of the training's result: it decides the BF16 rounding of
+// later weights), from tiles of kBiasRows rows that the block's threads load
+// ahead (one thread per column reading its column was latency-bound, 75 us
+// for 1024 rows).  With lr > 0 they then step the bias, and the other
+// blocks the weights with their BF16 copies and transposes.
+constexpr int kBiasRows = 64, kBiasCtas = 8;  // kGT * kBiasCtas = 256 columns at a time
+__global__ void __launch_bounds__(256) update_kernel(UpdateJobs u, float lr, float b1, float b2, float eps,
+                                                     float c1, float c2) {
+  __shared__ float tile[kBiasRows][kGT];
+  const int l = blockIdx.y, n_out = u.rows[l], n_in = u.cols[l];
+  if (blockIdx.x < kBiasCtas) {
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const float* G = u.G[l];
+    for (int c0 = blockIdx.x * kGT; c0 < n_out; c0 += kGT * kBiasCtas) {
+      const int col = c0 + tx;
+      float nx[kBiasRows / 8];
+#pragma unroll
+      for (int i = 0; i < kBiasRows / 8; ++i) nx[i] = col < n_out ? G[(size_t)(ty + 8 * i) * n_out + col] : 0.0f;
+      float s = 0.0f;
+      for (int r0 = 0; r0 < u.M; r0 += kBiasRows) {
+#pragma unroll
+        for (int i = 0; i < kBiasRows / 8; ++i) tile[ty + 8 * i][tx] = nx[i];
+        __syncthreads();
+        if (r0 + kBiasRows < u.M)
+#pragma unroll
+          for (int i = 0; i < kBiasRows / 8; ++i)
+            nx[i] = col < n_out ? G[(size_t)(r0 + kBiasRows + ty + 8 * i) * n_out + col] : 0.0f;
+        if (ty == 0)
+#pragma unroll 16
+          for (int r = 0; r < kBiasRows; ++r) s += tile[r][tx];
+        __syncthreads();
+      }
+      if (ty == 0 && col < n_out) {
+        u.gb[l][col] = s;
+        if (lr > 0.0f) adam_step(u.b[l], s, u.mb[l], u.vb[l], col, lr, b1, b2, eps, c1, c2);
+      }
+    }
+    return;
+  }
   const int64_t total = (int64_t)n_out * n_in;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    w[i] = wi;
-    if (w16) w16[i] = __float2bfloat16(wi);
-    if (wt16) {
-      const int64_t r = i / n_in, c = i % n_in;
-      wt16[c * n_out + r] = __float2bfloat16(wi);
-    }
-  }
-}
-
-// x (FP32, zeroed where mask <= 0 if a mask is given) as hi + lo BF16
-// parts: hi = bf16(x), lo = bf16(x - hi)
-__global__ void split_bf16_kernel(int64_t total, int cols, float* x, const __nv_bfloat16* mask,
-                                  int ldm, __nv_bfloat16* hi, __nv_bfloat16* lo) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    float v = x[i];
-    if (mask && !(__bfloat162float(mask[(i / cols) * ldm + i % cols]) > 0.0f)) {
-      v = 0.0f;
-      x[i] = 0.0f;
-    }
-    const __nv_bfloat16 h = __float2bfloat16(v);
-    hi[i] = h;
-    lo[i] = __float2bfloat16(v - __bfloat162float(h));
+  for (int64_t i = (blockIdx.x - kBiasCtas) * (int64_t)blockDim.x + threadIdx.x; i < total;
+       i += (int64_t)(gridDim.x - kBiasCtas) * blockDim.x) {
+    const float wi = adam_step(u.W[l], u.gW[l][i], u.mW[l], u.vW[l], i, lr, b1, b2, eps, c1, c2);
+    const __nv_bfloat16 h = __float2bfloat16(wi);
+    ((__nv_bfloat16*)u.W16[l])[i] = h;
+    const int64_t r = i / n_in, c = i % n_in;
+    ((__nv_bfloat16*)u.WT16[l])[c * n_out + r] = h;
   }
 }
 
@@ -453,41 +520,30 @@ cudaError_t launch_decode(int D, int64_t C, int Kmax, int O, const float* out, c
 }
 
 cudaError_t launch_loss_grad(int B, int O, int D, int Kmax, const float* out, const float* T,
-                             const float* Mk, float* G32, void* G16, double* loss,
-                             cudaStream_t s) {
-  const int64_t total = (int64_t)B * O;
-  const int g = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-  loss_grad_kernel<<<g, 256, 0, s>>>(B, O, mlp_SP(D), Kmax, out, T, Mk, G32,
-                                     (__nv_bfloat16*)G16, loss);
+                             const float* Mk, const GradOut& g, double* loss, cudaStream_t s) {
+  loss_grad_kernel<<<dim3((O + kGT - 1) / kGT, B / kGradRows), dim3(32, 8), 0, s>>>(B, O, mlp_SP(D), Kmax, out,
+                                                                                    T, Mk, g, loss);
   return cudaGetLastError();
 }
 
-cudaError_t launch_transpose_bf16(int R, int Cc, const void* in, int ldi, void* out, int ldo,
-                                  cudaStream_t s) {
-  dim3 grid((Cc + 31) / 32, (R + 31) / 32), block(32, 8);
-  transpose_bf16_kernel<<<grid, block, 0, s>>>(R, Cc, (const __nv_bfloat16*)in, ldi,
-                                               (__nv_bfloat16*)out, ldo);
+cudaError_t launch_grad_prep(int M, int Cc, const void* mask, const GradOut& g, cudaStream_t s) {
+  grad_prep_kernel<<<dim3((Cc + kGT - 1) / kGT, M / kGradRows), dim3(32, 8), 0, s>>>(
+      M, Cc, (const __nv_bfloat16*)mask, g);
   return cudaGetLastError();
 }
 
-cudaError_t launch_colsum(int R, int Cc, const void* G, int ld, int g_is_bf16, float* db,
-                          cudaStream_t s) {
-  const int g = (Cc + 127) / 128;
-  if (g_is_bf16)
-    colsum_kernel<__nv_bfloat16><<<g, 128, 0, s>>>(R, Cc, (const __nv_bfloat16*)G, ld, db);
-  else
-    colsum_kernel<float><<<g, 128, 0, s>>>(R, Cc, (const float*)G, ld, db);
+cudaError_t launch_transposes(int M, const TransposeJobs& t, cudaStream_t s) {
+  int most = 0;
+  for (int z = 0; z < 4; ++z) most = t.cols[z] > most ? t.cols[z] : most;
+  transposes_kernel<<<dim3((most + kGT - 1) / kGT, (M + kGT - 1) / kGT, 4), dim3(32, 8), 0, s>>>(M, t);
   return cudaGetLastError();
 }
 
-cudaError_t launch_adam(int n_out, int n_in, float* w, const float* g, float* m, float* v, float lr,
-                        int step, void* w16, void* wt16, cudaStream_t s) {
+cudaError_t launch_update(const UpdateJobs& u, float lr, int step, cudaStream_t s) {
   const float b1 = 0.9f, b2 = 0.999f;
-  const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);
-  const int64_t total = (int64_t)n_out * n_in;
-  const int nb = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-  adam_kernel<<<nb, 256, 0, s>>>(n_out, n_in, w, g, m, v, lr, b1, b2, 1e-8f, c1, c2,
-                                (__nv_bfloat16*)w16, (__nv_bfloat16*)wt16);
+  const float c1 = lr > 0.0f ? 1.0f - powf(b1, (float)step) : 1.0f;
+  const float c2 = lr > 0.0f ? 1.0f - powf(b2, (float)step) : 1.0f;
+  update_kernel<<<dim3(kBiasCtas + (lr > 0.0f ? 144 : 0), 4), 256, 0, s>>>(u, lr, b1, b2, 1e-8f, c1, c2);
   return cudaGetLastError();
 }
 
@@ -496,14 +552,6 @@ cudaError_t launch_cast_weights(int n_out, int n_in, const float* w, void* w16, 
   const int64_t total = (int64_t)n_out * n_in;
   const int g = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
   cast_weights_kernel<<<g, 256, 0, s>>>(n_out, n_in, w, (__nv_bfloat16*)w16, (__nv_bfloat16*)wt16);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_split_bf16(int64_t total, int cols, float* x, const void* mask, int ldm,
-                              void* hi, void* lo, cudaStream_t s) {
-  const int g = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-  split_bf16_kernel<<<g, 256, 0, s>>>(total, cols, x, (const __nv_bfloat16*)mask, ldm,
-                                      (__nv_bfloat16*)hi, (__nv_bfloat16*)lo);
   return cudaGetLastError();
 }
 

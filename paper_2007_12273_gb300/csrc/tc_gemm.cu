@@ -5,7 +5,10 @@
 //
 // A and B are BF16, "K-major" (row-major with K contiguous); accumulation is
 // FP32 in tensor memory (TMEM).  One CTA (4 warps) computes a 128 x BN tile,
-// walking K in chunks of 64 through an S-stage shared-memory ring:
+// walking K in chunks of 64 through an S-stage shared-memory ring (with a
+// second operand A2 it walks K again into a second accumulator and adds the
+// two in FP32: a gradient carried as two BF16 parts takes one launch and no
+// read of C):
 //   * thread 0 (warp 0) is the producer: per chunk one TMA tiled load
 //     (cp.async.bulk.tensor) of A (64 x 128) and one of B (64 x BN) with the
 //     128-byte swizzle, completing on the stage's "full" mbarrier;
@@ -111,18 +114,20 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[N]) {
 
 }  // namespace
 
-// BN: tile columns (32..256, a power of two); TMEM columns = BN rounded up
-// to a power of two >= 32; S: pipeline stages
-template <int BN, int S>
+// BN: tile columns (32..256, a power of two); S: pipeline stages; kTwo: a
+// second operand A2 with an accumulator of its own
+template <int BN, int S, bool kTwo>
 __global__ void __launch_bounds__(128) tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
+                                                      const __grid_constant__ CUtensorMap mapA2,
                                                       const __grid_constant__ CUtensorMap mapB,
                                                       int M, int N, int K,
                                                       const float* __restrict__ bias, int relu,
                                                       const __nv_bfloat16* __restrict__ mask,
                                                       int ldm, float* __restrict__ Cf,
                                                       __nv_bfloat16* __restrict__ Cb, int ldc,
-                                                      int accumulate, unsigned int* err) {
-  constexpr int TCOLS = BN <= 32 ? 32 : (BN <= 64 ? 64 : (BN <= 128 ? 128 : 256));
+                                                      unsigned int* err) {
+  constexpr int TCOLS = kTwo ? 2 * BN : BN;  // TMEM columns (a power of two, 32 .. 256)
+  static_assert(TCOLS >= 32 && TCOLS <= 256, "two CTAs of an SM share 512 columns");
   constexpr uint32_t IDESC = idesc_bf16(kBM, BN);
   constexpr uint32_t A_BYTES = kBM * kBK * 2, B_BYTES = BN * kBK * 2;
   constexpr uint32_t STAGE = A_BYTES + B_BYTES;  // a multiple of 1024
@@ -135,7 +140,7 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(const __grid_constant__ CU
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
-  const int nk = (K + kBK - 1) / kBK;
+  const int nk1 = (K + kBK - 1) / kBK, nk = kTwo ? 2 * nk1 : nk1;
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
@@ -172,8 +177,9 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(const __grid_constant__ CU
       const uint32_t fb = smem_u32(&full[st]);
       const uint32_t sa = smem_u32(smem + (size_t)st * STAGE);
       mbar_expect_tx(fb, STAGE);
-      tma_load_2d(sa, &mapA, kc * kBK, m0, fb);
-      tma_load_2d(sa + A_BYTES, &mapB, kc * kBK, n0, fb);
+      const int kx = (kc < nk1 ? kc : kc - nk1) * kBK;
+      tma_load_2d(sa, kc < nk1 ? &mapA : &mapA2, kx, m0, fb);
+      tma_load_2d(sa + A_BYTES, &mapB, kx, n0, fb);
       issued = kc + 1;
     }
     // on a time-out, wait (bounded) for the copies still in flight
@@ -196,10 +202,11 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(const __grid_constant__ CU
       for (int s = 0; s < kBK / 16; ++s) {
         const uint64_t ad = smem_desc_sw128(a0 + 32 * s);
         const uint64_t bd = smem_desc_sw128(b0 + 32 * s);
-        const uint32_t acc = (kc > 0 || s > 0) ? 1u : 0u;
+        const uint32_t acc = (kc % nk1 > 0 || s > 0) ? 1u : 0u;
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+                kc < nk1 ? tmem : tmem + BN),
             "l"(ad), "l"(bd), "r"(IDESC), "r"(acc));
       }
       asm volatile(
@@ -233,6 +240,12 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(const __grid_constant__ CU
     for (int c0 = 0; c0 < BN; c0 += 16) {
       float v[16];
       tmem_ld16<16>(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+      if constexpr (kTwo) {
+        float v2[16];
+        tmem_ld16<16>(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(BN + c0), v2);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[e] += v2[e];
+      }
       if (row >= M || n0 + c0 >= N) continue;
       const int cb = n0 + c0;
       if (cb + 16 <= N && vf && vb && vm) {
@@ -257,12 +270,7 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(const __grid_constant__ CU
           float4* cp = reinterpret_cast<float4*>(Cf + (size_t)row * ldc + cb);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            float4 o = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
-            if (accumulate) {
-              const float4 a = cp[q];
-              o.x += a.x; o.y += a.y; o.z += a.z; o.w += a.w;
-            }
-            cp[q] = o;
+            cp[q] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
           }
         }
         if (Cb) {
@@ -286,10 +294,7 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(const __grid_constant__ CU
         if (bias) x += bias[col];
         if (relu) x = fmaxf(x, 0.0f);
         if (mask && !(__bfloat162float(mask[(size_t)row * ldm + col]) > 0.0f)) x = 0.0f;
-        if (Cf) {
-          float* cp = Cf + (size_t)row * ldc + col;
-          *cp = accumulate ? *cp + x : x;
-        }
+        if (Cf) Cf[(size_t)row * ldc + col] = x;
         if (Cb) Cb[(size_t)row * ldc + col] = __float2bfloat16(x);
       }
     }
@@ -302,11 +307,13 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(const __grid_constant__ CU
 
 // ring depth: two stages (48 KB each for 128 x 256 tiles), so that two CTAs
 // share an SM (2 x 97 KB of shared memory, at most 2 x 256 TMEM columns)
-// and one's ring fill and epilogue overlap the other's MMAs
+// and one's ring fill and epilogue overlap the other's MMAs.  The narrow
+// tiles run with few CTAs (below), where a CTA's own ring has to cover the
+// load latency: six stages of 20 KB, four of 24 KB.
 template <int BN>
-constexpr int gemm_stages() { return 2; }
-
-size_t tc_gemm_smem(int bn) { return (size_t)(kBM + bn) * kBK * 2 * 2 + 1024; }
+constexpr int gemm_stages() { return BN == 32 ? 6 : (BN == 64 ? 4 : 2); }
+template <int BN>
+constexpr size_t gemm_smem() { return (size_t)(kBM + BN) * kBK * 2 * gemm_stages<BN>() + 1024; }
 
 namespace {
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -338,32 +345,44 @@ bool make_map(CUtensorMap* map, const void* base, int rows, int K, int ld, int b
 }
 }  // namespace
 
-cudaError_t launch_tc_gemm(const void* A, const void* B, int M, int N, int K, int lda, int ldb,
-                           const float* bias, int relu, const void* mask, int ldm, float* Cf,
-                           void* Cb, int ldc, unsigned int* err, cudaStream_t s, int accumulate) {
+cudaError_t launch_tc_gemm(const void* A, const void* A2, const void* B, int M, int N, int K, int lda,
+                           int ldb, const float* bias, int relu, const void* mask, int ldm, float* Cf,
+                           void* Cb, int ldc, unsigned int* err, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-  int bn = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 128 ? 128 : 256));
-  CUtensorMap mapA, mapB;
-  if (!make_map(&mapA, A, M, K, lda, kBM) || !make_map(&mapB, B, N, K, ldb, bn))
+  // the tile width covers N up to 256; where that leaves most SMs without a
+  // tile (a training batch's layers and weight gradients: 2 to 32 tiles) it
+  // is halved, as the loads of a long K, not the MMAs, set a tile's time:
+  // 256 x 256 x 1024 in hi + lo parts, 2 tiles of 256 columns against 16 of 32
+  int bn = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 128 || A2 ? 128 : 256));
+  const int64_t mt = (M + kBM - 1) / kBM;
+  while (bn > 32 && mt * ((N + bn - 1) / bn) < 76) bn >>= 1;
+  CUtensorMap mapA, mapA2, mapB;
+  if (!make_map(&mapA, A, M, K, lda, kBM) || !make_map(&mapA2, A2 ? A2 : A, M, K, lda, kBM) ||
+      !make_map(&mapB, B, N, K, ldb, bn))
     return cudaErrorInvalidValue;
-  // at least 80 KB of shared memory per CTA keeps two CTAs (2 x 256 TMEM
-  // columns) per SM at most, so a TMEM allocation never waits
-  size_t smem = tc_gemm_smem(bn);
-  if (smem < 80 * 1024) smem = 80 * 1024;
-  dim3 grid((M + kBM - 1) / kBM, (N + bn - 1) / bn);
-#define GM_TC_LAUNCH(BNV)                                                                        \
+  dim3 grid((unsigned)mt, (N + bn - 1) / bn);
+#define GM_TC_LAUNCH(BNV, TWO)                                                                   \
   {                                                                                              \
-    auto k = tc_gemm_kernel<BNV, gemm_stages<BNV>()>;                                             \
+    auto k = tc_gemm_kernel<BNV, gemm_stages<BNV>(), TWO>;                                        \
+    /* at least 80 KB of shared memory per CTA keeps two CTAs (2 x 256 TMEM columns) per SM at    \
+       most, so a TMEM allocation never waits */                                                 \
+    const size_t smem = gemm_smem<BNV>() < 80 * 1024 ? 80 * 1024 : gemm_smem<BNV>();             \
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
                                          (int)smem);                                             \
     if (e != cudaSuccess) return e;                                                              \
-    k<<<grid, 128, smem, s>>>(mapA, mapB, M, N, K, bias, relu, (const __nv_bfloat16*)mask, ldm, \
-                              Cf, (__nv_bfloat16*)Cb, ldc, accumulate, err);                     \
+    k<<<grid, 128, smem, s>>>(mapA, mapA2, mapB, M, N, K, bias, relu, (const __nv_bfloat16*)mask, \
+                              ldm, Cf, (__nv_bfloat16*)Cb, ldc, err);                             \
   }
-  if (bn == 32) GM_TC_LAUNCH(32)
-  else if (bn == 64) GM_TC_LAUNCH(64)
-  else if (bn == 128) GM_TC_LAUNCH(128)
-  else GM_TC_LAUNCH(256)
+  if (A2) {
+    if (bn == 32) GM_TC_LAUNCH(32, true)
+    else if (bn == 64) GM_TC_LAUNCH(64, true)
+    else GM_TC_LAUNCH(128, true)
+  } else {
+    if (bn == 32) GM_TC_LAUNCH(32, false)
+    else if (bn == 64) GM_TC_LAUNCH(64, false)
+    else if (bn == 128) GM_TC_LAUNCH(128, false)
+    else GM_TC_LAUNCH(256, false)
+  }
 #undef GM_TC_LAUNCH
   return cudaGetLastError();
 }
