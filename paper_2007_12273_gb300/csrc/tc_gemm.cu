@@ -219,6 +219,10 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(const __grid_constant__ CU
             smem_u32(&done))
         : "memory");
   }
+  // the other lanes of the producer's and the issuer's warps wait here, not
+  // at the barrier below: a lane suspended in its try_wait would suspend its
+  // warp, and with it the role's thread, for a microsecond or more per chunk
+  __syncwarp();
   // the accumulator is complete once the last commit arrives (the commit
   // tracks every earlier MMA of this thread)
   if (!mbar_wait(smem_u32(&done), 0u)) {
