@@ -31,6 +31,19 @@ __device__ __forceinline__ bool equal_weights(const double* alpha, int64_t o, in
   return __all_sync(0xffffffffu, same);
 }
 
+// k = round(xi 2^53) - 2^52 of an FP64 xi in [0, 1), from its bits
+__device__ __forceinline__ long long frac_k(double xi) {
+  // xi = m 2^(e - 1075) (m with its implicit bit)
+  const unsigned long long u = (unsigned long long)__double_as_longlong(xi);
+  const int e = (int)((u >> 52) & 0x7FFull);
+  const long long m = (long long)((u & ((1ull << 52) - 1ull)) | (e ? (1ull << 52) : 0ull));
+  const int sh = (e ? e : 1) - 1022;  // xi 2^53 = m 2^sh, sh <= 0
+  long long rr = 0;
+  if (sh == 0) rr = m;
+  else if (sh > -60) rr = (m + (1ll << (-sh - 1))) >> (-sh);
+  return rr - (1ll << 52);
+}
+
 // cell j's record r; same = equal_weights(...) for 0 < n <= kFixMaxN
 __device__ __forceinline__ void deposit_cell(int64_t j, int64_t o, int64_t n, const double* x,
                                              const double* alpha, double inv_dx, int order,
@@ -48,16 +61,7 @@ __device__ __forceinline__ void deposit_cell(int64_t j, int64_t o, int64_t n, co
     __int128 k1 = 0;
 #pragma unroll 2
     for (int64_t p = lane; p < n; p += 32) {
-      const double xi = cell_frac(x[o + p], jd, inv_dx);
-      // xi = m 2^(e - 1075) (m with its implicit bit), k = round(xi 2^53) - 2^52
-      const unsigned long long u = (unsigned long long)__double_as_longlong(xi);
-      const int e = (int)((u >> 52) & 0x7FFull);
-      const long long m = (long long)((u & ((1ull << 52) - 1ull)) | (e ? (1ull << 52) : 0ull));
-      const int sh = (e ? e : 1) - 1022;  // xi 2^53 = m 2^sh, sh <= 0
-      long long rr = 0;
-      if (sh == 0) rr = m;
-      else if (sh > -60) rr = (m + (1ll << (-sh - 1))) >> (-sh);
-      const long long k = rr - (1ll << 52);
+      const long long k = frac_k(cell_frac(x[o + p], jd, inv_dx));
       if (order == 1) {
         k0l += k < 0 ? -k : 0;
         k1 += (__int128)(k > 0 ? k : 0);
@@ -82,27 +86,67 @@ __device__ __forceinline__ void deposit_cell(int64_t j, int64_t o, int64_t n, co
     if (lane < kDepWords) r[lane] = wv;
     return;
   }
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-  for (int64_t p = lane; p < n; p += 32) {
-    const double sx = cell_frac(x[o + p], jd, inv_dx) - 0.5;
-    const double al = alpha ? alpha[o + p] : 1.0;
-    if (order == 1) {
-      a0 += al;
-      a1 = sx < 0.0 ? fma(-al, sx, a1) : a1;
-      a2 = sx > 0.0 ? fma(al, sx, a2) : a2;
+  // otherwise by chunks of kSumChunk particles: in fixed point (see
+  // kScaleBits), or in FP64 where a weight is not finite
+  ChunkSum tot;  // sum t on lane t < 3
+  for (int64_t c0 = o; c0 < o + n; c0 += kSumChunk) {
+    const int m = (int)(o + n - c0 < kSumChunk ? o + n - c0 : kSumChunk);
+    int ea = 0;
+#pragma unroll 4
+    for (int p = lane; p < m; p += 32) ea = max(ea, exp_field(alpha ? alpha[c0 + p] : 1.0));
+    ea = warp_imax(ea);
+    double mine;
+    if (exp_finite(ea, 0.0)) {
+      const int eq = scale_exp(ea, 0.0);
+      const TermShift sh(m, 62);
+      long long s0 = 0, s1 = 0, s2 = 0;  // units of 2^(eq + sh.s)
+#pragma unroll 2
+      for (int p = lane; p < m; p += 32) {
+        const long long k = frac_k(cell_frac(x[c0 + p], jd, inv_dx));
+        const long long a = fixq(alpha ? alpha[c0 + p] : 1.0, eq), X = k << 11;  // s = X 2^-64
+        const long long as = __mul64hi(a, X);
+        s0 += sh(a);
+        if (order == 1) {
+          const long long t = sh(as);
+          s1 -= k < 0 ? t : 0;
+          s2 += k > 0 ? t : 0;
+        } else {
+          s1 += sh(as);
+          s2 += sh(__mul64hi(as, X));
+        }
+      }
+      __int128 t0 = s0, t1 = s1, t2 = s2;
+#pragma unroll
+      for (int q = 16; q > 0; q >>= 1) {
+        t0 += shfl_xor_i128(t0, q);
+        t1 += shfl_xor_i128(t1, q);
+        t2 += shfl_xor_i128(t2, q);
+      }
+      mine = i128_to_f64(lane == 0 ? t0 : (lane == 1 ? t1 : t2), eq + sh.s);
     } else {
-      const double as = al * sx;
-      a0 += al;
-      a1 += as;
-      a2 = fma(as, sx, a2);
+      double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+      for (int p = lane; p < m; p += 32) {
+        const double sx = cell_frac(x[c0 + p], jd, inv_dx) - 0.5;
+        const double al = alpha ? alpha[c0 + p] : 1.0;
+        if (order == 1) {
+          a0 += al;
+          a1 = sx < 0.0 ? fma(-al, sx, a1) : a1;
+          a2 = sx > 0.0 ? fma(al, sx, a2) : a2;
+        } else {
+          const double as = al * sx;
+          a0 += al;
+          a1 += as;
+          a2 = fma(as, sx, a2);
+        }
+      }
+      a0 = warp_sum(a0);
+      a1 = warp_sum(a1);
+      a2 = warp_sum(a2);
+      mine = lane == 0 ? a0 : (lane == 1 ? a1 : a2);
     }
+    tot.add(mine, c0 == o);
   }
-  a0 = warp_sum(a0);
-  a1 = warp_sum(a1);
-  a2 = warp_sum(a2);
-  long long wv = __double_as_longlong(a0);
-  wv = lane == 1 ? __double_as_longlong(a1) : wv;
-  wv = lane == 2 ? __double_as_longlong(a2) : wv;
+  long long wv = __double_as_longlong(tot.value());
   wv = lane == 5 ? -1ll : wv;
   if (lane < kDepWords) r[lane] = wv;
 }

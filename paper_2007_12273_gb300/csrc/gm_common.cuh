@@ -139,17 +139,112 @@ __device__ __forceinline__ long long fixq(float v, int eq) {
   return (u >> 31) ? -r : r;
 }
 
+// d / 2^eq rounded to the nearest integer (ties away from zero), from the
+// bit pattern of an FP64 d with |d| < 2^(eq + 62)
+__device__ __forceinline__ long long fixq(double d, int eq) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+  const int e = (int)((u >> 52) & 0x7FFull);
+  const long long m = (long long)((u & ((1ull << 52) - 1ull)) | (e ? (1ull << 52) : 0ull));
+  const int sh = (e ? e : 1) - 1075 - eq;  // d = m 2^(e - 1075)
+  long long r = 0;
+  if (sh >= 0) r = m << (sh < 9 ? sh : 9);
+  else if (sh > -60) r = (m + (1ll << (-sh - 1))) >> (-sh);
+  return (u >> 63) ? -r : r;
+}
+
+// Weighted sums in fixed point.  The weights and the velocities (or the
+// offsets) of a cell are taken to kScaleBits bits below the largest's
+// exponent, products are the high halves of 64 x 64-bit products, and every
+// term is rounded so that a lane's terms fit in 64 bits.  A cell goes by chunks
+// of kSumChunk particles (64 terms a lane, rounded to 2^-56 of the largest
+// product's bound), whose sums add up in FP64 with the additions' errors.
+// FP64 sums round at every addition, to 2^-53 of the partial sum.  An FP64
+// operation takes the SM's pipe 19 cycles, in which it issues some 70 integer
+// instructions: a product and its sum take about 15.
+constexpr int kScaleBits = 62;
+constexpr int kSumChunk = 2048;
+// a sum of chunk sums with the errors of its additions (Knuth's two-sum)
+struct ChunkSum {
+  double s = 0.0, e = 0.0;
+  __device__ __forceinline__ void add(double v, bool first) {
+    if (first) {
+      s = v;
+      return;
+    }
+    const double t = s + v, z = t - s;
+    e += (s - (t - z)) + (v - z);
+    s = t;
+  }
+  // the errors of a sum that is not finite are NaN
+  __device__ __forceinline__ double value() const { return isfinite(s) ? s + e : s; }
+};
+// biased exponent, and the exponent eq of fixq for values up to it
+__device__ __forceinline__ int exp_field(double d) { return (int)((__double_as_longlong(d) >> 52) & 0x7FF); }
+__device__ __forceinline__ int exp_field(float f) { return (int)((__float_as_uint(f) >> 23) & 0xFFu); }
+__device__ __forceinline__ int scale_exp(int emax, double) { return (emax ? emax : 1) - 1022 - kScaleBits; }
+__device__ __forceinline__ int scale_exp(int emax, float) { return (emax ? emax : 1) - 126 - kScaleBits; }
+__device__ __forceinline__ bool exp_finite(int emax, double) { return emax < 0x7FF; }
+__device__ __forceinline__ bool exp_finite(int emax, float) { return emax < 0xFF; }
+// rounding shift of terms below 2^62 of which a lane adds up to ceil(n / 32)
+struct TermShift {
+  int s;
+  long long half;
+  // bits: the terms are below 2^bits
+  __device__ __forceinline__ TermShift(int64_t n, int bits) {
+    const int terms = (int)((n + 31) >> 5);
+    s = (terms > 1 ? 32 - __clz(terms - 1) : 0) - (62 - bits);
+    s = s > 0 ? s : 0;
+    half = s > 0 ? 1ll << (s - 1) : 0;
+  }
+  __device__ __forceinline__ long long operator()(long long v) const { return (v + half) >> s; }
+};
+__device__ __forceinline__ int warp_imax(int v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
 __device__ __forceinline__ __int128 shfl_xor_i128(__int128 x, int b) {
   const long long lo = __shfl_xor_sync(0xffffffffu, (long long)(unsigned long long)x, b);
   const long long hi = __shfl_xor_sync(0xffffffffu, (long long)(x >> 64), b);
   return ((__int128)hi << 64) | (__int128)(unsigned long long)lo;
 }
 
-// a 128-bit integer times 2^e as the nearest-ish double (two roundings)
+// warp sums of NP 64-bit integers in 128 bits by recursive halving: lane l
+// ends with the total of value warp_rs_index<NP>(l)
+template <int NP>
+__device__ __forceinline__ __int128 warp_rs_i128(const long long (&v)[NP], int lane) {
+  static_assert(NP == 4 || NP == 16, "4 or 16 values");
+  constexpr int LV = NP == 4 ? 2 : 4;
+  __int128 w[NP / 2];
+  bool up = (lane & 16) != 0;
+#pragma unroll
+  for (int i = 0; i < NP / 2; ++i)
+    w[i] = (__int128)(up ? v[i + NP / 2] : v[i]) +
+           (__int128)__shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + NP / 2], 16);
+#pragma unroll
+  for (int lv = 1; lv < LV; ++lv) {
+    const int h2 = NP >> (lv + 1), b = 16 >> lv;
+    up = (lane & b) != 0;
+#pragma unroll
+    for (int i = 0; i < h2; ++i) {
+      const __int128 send = up ? w[i] : w[i + h2];
+      w[i] = (up ? w[i + h2] : w[i]) + shfl_xor_i128(send, b);
+    }
+  }
+#pragma unroll
+  for (int b = 16 >> LV; b >= 1; b >>= 1) w[0] += shfl_xor_i128(w[0], b);
+  return w[0];
+}
+
+// a 128-bit integer times 2^e as the nearest-ish double (two roundings), from
+// its sign and magnitude: a small negative sum's low word as it stands is near
+// 2^64, and its rounding would take 10 bits off the sum
 __device__ __forceinline__ double i128_to_f64(__int128 x, int e) {
-  const long long hi = (long long)(x >> 64);
-  const unsigned long long lo = (unsigned long long)x;
-  return ldexp(fma((double)hi, 18446744073709551616.0, (double)lo), e);
+  const unsigned __int128 m = x < 0 ? -(unsigned __int128)x : (unsigned __int128)x;
+  const unsigned long long hi = (unsigned long long)(m >> 64), lo = (unsigned long long)m;
+  const double r = ldexp(fma((double)hi, 18446744073709551616.0, (double)lo), e);
+  return x < 0 ? -r : r;
 }
 
 __device__ __forceinline__ float warp_max(float v) {

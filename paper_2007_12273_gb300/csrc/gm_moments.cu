@@ -4,22 +4,6 @@
 
 namespace gmcr {
 
-// Block-wide FP64 sum of NV values held per thread; result valid in thread 0.
-template <int NT, int NV>
-__device__ __forceinline__ void block_sum_to0(double (&v)[NV], double (*red)[NV]) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
-  if (lane == 0)
-#pragma unroll
-    for (int i = 0; i < NV; ++i) red[w][i] = v[i];
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int q = 1; q < NT / 32; ++q)
-#pragma unroll
-      for (int i = 0; i < NV; ++i) v[i] += red[q][i];
-}
-
 // Per-cell partial deposits: part[j] = sum_{p in j} alpha_p S(x_i - x_p)
 // for i = j-1, j, j+1 (alpha = NULL means unit weights).  With s = xi - 1/2
 // (xi the position inside the cell) the quadratic B-spline weights are
@@ -88,44 +72,134 @@ __global__ void deposit_combine_kernel(int64_t C, const long long* rec, int orde
   }
 }
 
-// W, p, M2 (upper triangle), E of each cell's particles
-template <int D, int NT, typename VT>
-__global__ void __launch_bounds__(NT) moments_kernel(int64_t C, int64_t n, const int64_t* cell_off,
-                                                     const VT* v, const double* alpha, double* W,
-                                                     double* p, double* M2, double* E) {
+// W, p, M2 (upper triangle), E of each cell's particles, one warp per cell, by
+// chunks of kSumChunk particles.  A chunk of finite particles takes fixed-point
+// sums (see kScaleBits): a pass for the largest exponents, then alpha, alpha v
+// and alpha v v^T on the integer pipe, converted to FP64 a sum per lane.  A
+// chunk whose largest weight and largest velocity belong to different particles
+// so far apart that the bound of alpha v or alpha v^2 exceeds the largest one
+// 2^kSlack times (its small terms would lose bits) sums in FP64 (13 operations
+// a particle for D = 3).  A CTA per cell with 28 FP64 operations a particle and
+// FP64 sums over its warps took 2.83 ms for 65536 3V cells of 572 weighted
+// particles (FP64 pipe); moments and deposit together went from 3.57 to 1.36 ms
+// (1.1 GB: issue slots bound both now).  Six CTAs an SM (80 registers) hide the
+// loads and the reductions better than five (95).  E = tr(M2) / 2.
+constexpr int kSlack = 4;
+template <int D, int NW, typename VT>
+__global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_t C, int64_t n, const int64_t* cell_off,
+                                                          const VT* v, const double* alpha, double* W,
+                                                          double* p, double* M2, double* E) {
   constexpr int NM = D * (D + 1) / 2;
-  constexpr int NV = 1 + D + NM + 1;
-  __shared__ double red[NT / 32][NV];
-  for (int64_t j = blockIdx.x; j < C; j += gridDim.x) {
-    const int64_t o = cell_off[j], cnt = cell_off[j + 1] - o;
-    double acc[NV];
+  constexpr int NS = 1 + D + NM;
+  constexpr int NP = NS <= 4 ? 4 : 16;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int64_t j = (int64_t)blockIdx.x * NW + wid; j < C; j += (int64_t)gridDim.x * NW) {
+    const int64_t o = cell_off[j], end = cell_off[j + 1];
+    ChunkSum tot;  // sum t on lane t < NS
+    for (int64_t c0 = o; c0 < end; c0 += kSumChunk) {
+      const int cnt = (int)(end - c0 < kSumChunk ? end - c0 : kSumChunk);
+      const double* al = alpha + c0;
+      const VT* vj = v ? v + c0 : nullptr;  // no velocities: the weights' sum alone
+      // the largest exponents
+      int ea = 0, ev[D], e1[D], e2[D];  // of alpha, v, alpha v, alpha v^2
 #pragma unroll
-    for (int i = 0; i < NV; ++i) acc[i] = 0.0;
-    for (int64_t q = threadIdx.x; q < cnt; q += NT) {
-      const double al = alpha[o + q];
-      double vv[D];
+      for (int d = 0; d < D; ++d) ev[d] = e1[d] = e2[d] = 0;
+#pragma unroll 4
+      for (int q = lane; q < cnt; q += 32) {
+        const int xa = exp_field(al[q]);
+        ea = max(ea, xa);
+        if (vj)
 #pragma unroll
-      for (int d = 0; d < D; ++d) vv[d] = (double)v[(int64_t)d * n + o + q];
-      acc[0] += al;
-      int t = 1 + D;
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        acc[1 + a] += al * vv[a];
-        acc[NV - 1] += 0.5 * al * vv[a] * vv[a];
-#pragma unroll
-        for (int b = a; b < D; ++b, ++t) acc[t] += al * vv[a] * vv[b];
+          for (int d = 0; d < D; ++d) {
+            const int xv = exp_field(vj[(int64_t)d * n + q]);
+            ev[d] = max(ev[d], xv);
+            e1[d] = max(e1[d], xa + xv);
+            e2[d] = max(e2[d], xa + 2 * xv);
+          }
       }
+      ea = warp_imax(ea);
+      bool fixed = exp_finite(ea, 0.0);
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        ev[d] = warp_imax(ev[d]);
+        fixed = fixed && exp_finite(ev[d], VT(0)) && ea + ev[d] - warp_imax(e1[d]) <= kSlack &&
+                ea + 2 * ev[d] - warp_imax(e2[d]) <= kSlack;
+      }
+      double mine;
+      if (fixed) {
+        const int qa = scale_exp(ea, 0.0);
+        int qv[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) qv[d] = scale_exp(ev[d], VT(0));
+        const TermShift s0(cnt, 62), s1(cnt, 60);
+        // units: 2^(qa + s0.s); 2^(qa + qv + 64 + s1.s); 2^(qa + qv + qv' + 126 + s1.s)
+        long long s[NP];
+#pragma unroll
+        for (int t = 0; t < NP; ++t) s[t] = 0;
+        for (int q = lane; q < cnt; q += 32) {
+          const long long a = fixq(al[q], qa);
+          s[0] += s0(a);
+          if (vj) {
+            long long vq[D], av[D];
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+              vq[d] = fixq(vj[(int64_t)d * n + q], qv[d]);
+              av[d] = __mul64hi(a, vq[d]);  // below 2^60, units of 2^(qa + qv + 64)
+              s[1 + d] += s1(av[d]);
+            }
+            int t = 1 + D;
+#pragma unroll
+            for (int x = 0; x < D; ++x)
+#pragma unroll
+              for (int y = x; y < D; ++y, ++t) s[t] += s1(__mul64hi(av[x] << 2, vq[y]));
+          }
+        }
+        const int i = warp_rs_index<NP>(lane);
+        int unit = qa + s0.s, t = 1 + D;
+#pragma unroll
+        for (int d = 0; d < D; ++d) unit = i == 1 + d ? qa + qv[d] + 64 + s1.s : unit;
+#pragma unroll
+        for (int x = 0; x < D; ++x)
+#pragma unroll
+          for (int y = x; y < D; ++y, ++t) unit = i == t ? qa + qv[x] + qv[y] + 126 + s1.s : unit;
+        mine = i128_to_f64(warp_rs_i128<NP>(s, lane), unit);
+      } else {
+        double acc[NP];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) acc[i] = 0.0;
+        for (int q = lane; q < cnt; q += 32) {
+          const double a = al[q];
+          acc[0] += a;
+          if (vj) {
+            double vv[D];
+#pragma unroll
+            for (int d = 0; d < D; ++d) vv[d] = to_f64(vj[(int64_t)d * n + q]);
+            int t = 1 + D;
+#pragma unroll
+            for (int x = 0; x < D; ++x) {
+              const double ax = a * vv[x];
+              acc[1 + x] += ax;
+#pragma unroll
+              for (int y = x; y < D; ++y, ++t) acc[t] = fma(ax, vv[y], acc[t]);
+            }
+          }
+        }
+        warp_rs_d<NP>(acc, lane);
+        mine = acc[0];
+      }
+      mine = __shfl_sync(0xffffffffu, mine, warp_rs_lane<NP>(lane & (NP - 1)));
+      tot.add(mine, c0 == o);
     }
-    block_sum_to0<NT, NV>(acc, red);
-    if (threadIdx.x == 0) {
-      if (W) W[j] = acc[0];
-      if (p)
-        for (int a = 0; a < D; ++a) p[j * D + a] = acc[1 + a];
-      if (M2)
-        for (int t = 0; t < NM; ++t) M2[j * NM + t] = acc[1 + D + t];
-      if (E) E[j] = acc[NV - 1];
+    const double mine = tot.value();
+    if (W && lane == 0) W[j] = mine;
+    if (p && lane >= 1 && lane <= D) p[j * D + lane - 1] = mine;
+    if (M2 && lane > D && lane < NS) M2[j * NM + lane - 1 - D] = mine;
+    if (E) {
+      double tr = __shfl_sync(0xffffffffu, mine, 1 + D);
+      if (D == 3)
+        tr = (tr + __shfl_sync(0xffffffffu, mine, 7 < NS ? 7 : 0)) + __shfl_sync(0xffffffffu, mine, 9 < NS ? 9 : 0);
+      if (lane == 0) E[j] = 0.5 * tr;
     }
-    __syncthreads();
   }
 }
 
@@ -192,17 +266,18 @@ cudaError_t launch_moments(int D, int64_t C, int64_t n, const int64_t* cell_off,
                            int v_f64, const double* alpha, double* W, double* p, double* M2,
                            double* E, cudaStream_t s) {
   if (C == 0) return cudaSuccess;
-  const int g = grid_for(C, 152 * 16);
+  constexpr int NW = 4;
+  const int g = grid_for((C + NW - 1) / NW, 152 * 16);
   if (D == 1) {
     if (v_f64)
-      moments_kernel<1, 128, double><<<g, 128, 0, s>>>(C, n, cell_off, (const double*)v, alpha, W, p, M2, E);
+      moments_kernel<1, NW, double><<<g, NW * 32, 0, s>>>(C, n, cell_off, (const double*)v, alpha, W, p, M2, E);
     else
-      moments_kernel<1, 128, float><<<g, 128, 0, s>>>(C, n, cell_off, (const float*)v, alpha, W, p, M2, E);
+      moments_kernel<1, NW, float><<<g, NW * 32, 0, s>>>(C, n, cell_off, (const float*)v, alpha, W, p, M2, E);
   } else {
     if (v_f64)
-      moments_kernel<3, 128, double><<<g, 128, 0, s>>>(C, n, cell_off, (const double*)v, alpha, W, p, M2, E);
+      moments_kernel<3, NW, double><<<g, NW * 32, 0, s>>>(C, n, cell_off, (const double*)v, alpha, W, p, M2, E);
     else
-      moments_kernel<3, 128, float><<<g, 128, 0, s>>>(C, n, cell_off, (const float*)v, alpha, W, p, M2, E);
+      moments_kernel<3, NW, float><<<g, NW * 32, 0, s>>>(C, n, cell_off, (const float*)v, alpha, W, p, M2, E);
   }
   return cudaGetLastError();
 }

@@ -376,18 +376,6 @@ __device__ __forceinline__ int fix_exponent(float b, int bits) {
   const int eb = (int)((__float_as_uint(b) >> 23) & 0xFFu);
   return (eb ? eb - 127 : -126) + 1 - bits;
 }
-// d / 2^eq rounded to the nearest integer (ties away from zero), from the
-// bit pattern of an FP64 d with |d| < 2^(eq + 54)
-__device__ __forceinline__ long long fixq_d(double d, int eq) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(d);
-  const int e = (int)((u >> 52) & 0x7FFull);
-  const long long m = (long long)((u & ((1ull << 52) - 1ull)) | (e ? (1ull << 52) : 0ull));
-  const int sh = (e ? e : 1) - 1075 - eq;  // d = m 2^(e - 1075)
-  long long r = 0;
-  if (sh >= 0) r = m << (sh < 10 ? sh : 10);
-  else if (sh > -60) r = (m + (1ll << (-sh - 1))) >> (-sh);
-  return (u >> 63) ? -r : r;
-}
 // The fixed-point plan of a cell in the warp's RecCell: the exponents eq and
 // (several components) dzq[k] = dz_k / 2^eq.  One component: f alone, kFixBits
 // bits, so that a lane's kFixMaxN / 32 = 512 terms (0.96 x 2^54 each) stay
@@ -416,7 +404,7 @@ __device__ __forceinline__ bool fix_plan(const RecCell<D>& rc, int64_t n, int la
   if (!__all_sync(0xffffffffu, ok)) return false;
   if (lane < K)
 #pragma unroll
-    for (int d = 0; d < D; ++d) dzq[lane][d] = fixq_d(rc.dz[lane][d], eq[d]);
+    for (int d = 0; d < D; ++d) dzq[lane][d] = fixq(rc.dz[lane][d], eq[d]);
   __syncwarp();
   return true;
 }
