@@ -44,6 +44,41 @@ __device__ __forceinline__ long long frac_k(double xi) {
   return rr - (1ll << 52);
 }
 
+// a lane's sums of k and k^2 (quadratic B-spline) or of the CIC parts
+// max(-k, 0) and max(k, 0), |k| <= 2^52, over up to kFixMaxN / 32 = 512
+// particles: k = h 2^27 + l has |h| <= 2^25, so that SplitSum's parts stay
+// below 2^63 for 512 terms
+struct DepSums {
+  long long k0 = 0;
+  SplitSum q;
+  __device__ __forceinline__ void add(long long k, int order) {
+    if (order == 1) {
+      k0 += k < 0 ? -k : 0;
+      q.ll += k > 0 ? k : 0;
+    } else {
+      k0 += k;
+      q.add_square(SplitInt(k));
+    }
+  }
+  // the equal-weight record r (weight bits wb) of the warp's cell
+  __device__ __forceinline__ void put(long long wb, int64_t n, int order, long long* r, int lane) const {
+    __int128 s0 = (__int128)k0, s1 = order == 1 ? (__int128)q.ll : q.total_square();
+#pragma unroll
+    for (int b = 16; b > 0; b >>= 1) {
+      s0 += shfl_xor_i128(s0, b);
+      s1 += shfl_xor_i128(s1, b);
+    }
+    // lanes 0-5 write the record's words
+    long long wv = (long long)(unsigned long long)s0;
+    wv = lane == 1 ? (long long)(s0 >> 64) : wv;
+    wv = lane == 2 ? (long long)(unsigned long long)s1 : wv;
+    wv = lane == 3 ? (long long)(s1 >> 64) : wv;
+    wv = lane == 4 ? wb : wv;
+    wv = lane == 5 ? (long long)n : wv;
+    if (lane < kDepWords) r[lane] = wv;
+  }
+};
+
 // cell j's record r; same = equal_weights(...) for 0 < n <= kFixMaxN
 __device__ __forceinline__ void deposit_cell(int64_t j, int64_t o, int64_t n, const double* x,
                                              const double* alpha, double inv_dx, int order,
@@ -55,35 +90,10 @@ __device__ __forceinline__ void deposit_cell(int64_t j, int64_t o, int64_t n, co
   // position xi in [0, 1); the weight multiplies the sums once
   if (n > 0 && n <= kFixMaxN && same) {
     const long long wb = alpha ? __double_as_longlong(alpha[o]) : __double_as_longlong(1.0);
-    // a lane sums at most kFixMaxN / 32 = 512 values of |k| <= 2^52: the
-    // linear sum fits in 64 bits, the squares take 128
-    long long k0l = 0;
-    __int128 k1 = 0;
+    DepSums t;
 #pragma unroll 2
-    for (int64_t p = lane; p < n; p += 32) {
-      const long long k = frac_k(cell_frac(x[o + p], jd, inv_dx));
-      if (order == 1) {
-        k0l += k < 0 ? -k : 0;
-        k1 += (__int128)(k > 0 ? k : 0);
-      } else {
-        k0l += k;
-        k1 += (__int128)k * (__int128)k;
-      }
-    }
-    __int128 k0 = (__int128)k0l;
-#pragma unroll
-    for (int q = 16; q > 0; q >>= 1) {
-      k0 += shfl_xor_i128(k0, q);
-      k1 += shfl_xor_i128(k1, q);
-    }
-    // lanes 0-5 write the record's words
-    long long wv = (long long)(unsigned long long)k0;
-    wv = lane == 1 ? (long long)(k0 >> 64) : wv;
-    wv = lane == 2 ? (long long)(unsigned long long)k1 : wv;
-    wv = lane == 3 ? (long long)(k1 >> 64) : wv;
-    wv = lane == 4 ? wb : wv;
-    wv = lane == 5 ? (long long)n : wv;
-    if (lane < kDepWords) r[lane] = wv;
+    for (int64_t p = lane; p < n; p += 32) t.add(frac_k(cell_frac(x[o + p], jd, inv_dx)), order);
+    t.put(wb, n, order, r, lane);
     return;
   }
   // otherwise by chunks of kSumChunk particles: in fixed point (see

@@ -28,16 +28,6 @@
 
 namespace gmcr {
 
-// first lane holding the total of value q after warp_rs_d<NP>
-template <int NP>
-__device__ __forceinline__ int warp_rs_lane(int q) {
-  int l = 0;
-#pragma unroll
-  for (int lv = 0; (NP >> lv) > 1; ++lv)
-    if (q & (NP >> (lv + 1))) l |= 16 >> lv;
-  return l;
-}
-
 // The Cholesky floor test of a symmetric D x D matrix (upper triangle S),
 // by its L~ diag(p) L~^T pivots p_i (the squared Cholesky diagonal, FP64,
 // two reciprocals and no square root): every p_i sc2_i > fl and p_i <
@@ -77,61 +67,105 @@ __device__ __forceinline__ bool ldl_floor(const double* S, const double* sc2, do
 // once per cell -- no FP64 arithmetic per particle, where GB300's FP64 pipe
 // (1/64 of the FP32 rate) bounds the FP64 sums.
 // ---------------------------------------------------------------------------
-// the 128-bit sums [sum d (D), sum d d^T (upper, NM)] of an equal-weight
-// cell (n particles, velocities v[d * ldv + p], shift = the first particle)
-// in units of 2^eq_d (2^(eq_x + eq_y) for the products), on the integer
-// pipe, lane-parallel over particles; every lane returns them.  Returns
-// false (nothing written) when a velocity is not finite.
-template <int D>
-__device__ bool fixed_sums(const float* __restrict__ v, int64_t ldv, int n, int lane,
-                           __int128 (&s1)[D], __int128 (&s2)[D * (D + 1) / 2], int (&eq)[D]) {
-  constexpr int NM = D * (D + 1) / 2;
-  // the largest biased exponent per dimension
-  int emax[D];
+// Particles go by batches of kBatch a lane whose loads are issued together
+// (indexes past the end read the last particle again).
+constexpr int kBatch = 4;
+// A warp's scan of a cell before its velocity sums, one pass over the weights,
+// the velocities and (kDep) the positions: whether the weights are equal bit
+// for bit, the largest magnitude bits per dimension, and the lane's deposit
+// sums as if the weights were equal.
+template <int D, bool kDep>
+__device__ __forceinline__ bool k1_scan(const double* __restrict__ alpha, const float* __restrict__ v, int64_t ldv,
+                                        const double* __restrict__ x, double jd, double inv_dx, int order, int n,
+                                        int lane, int (&vmax)[D], DepSums& dep) {
+  const long long wb = __double_as_longlong(alpha[0]);
+  bool same = true;
 #pragma unroll
-  for (int d = 0; d < D; ++d) emax[d] = 0;
-#pragma unroll 4
-  for (int p = lane; p < n; p += 32)
+  for (int d = 0; d < D; ++d) vmax[d] = 0;
+  for (int p = lane; p < n; p += 32 * kBatch) {
+    double wt[kBatch], xp[kBatch];
+    float vp[kBatch][D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) emax[d] = max(emax[d], (int)((__float_as_uint(v[d * ldv + p]) >> 23) & 0xFFu));
-  bool ok = true;
+    for (int u = 0; u < kBatch; ++u) {
+      const int q = min(p + 32 * u, n - 1);
+      wt[u] = __ldcs(alpha + q);  // read once: the velocities are to stay in L1
+      if (kDep) xp[u] = __ldcs(x + q);
 #pragma unroll
-  for (int d = 0; d < D; ++d) {
+      for (int d = 0; d < D; ++d) vp[u][d] = v[d * ldv + q];
+    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) emax[d] = max(emax[d], __shfl_xor_sync(0xffffffffu, emax[d], o));
-    ok = ok && emax[d] < 255;
-    eq[d] = (emax[d] ? emax[d] - 127 : -126) + 1 - kFixBits;
+    for (int u = 0; u < kBatch; ++u) {
+      same &= __double_as_longlong(wt[u]) == wb;
+#pragma unroll
+      for (int d = 0; d < D; ++d) vmax[d] = max(vmax[d], (int)(__float_as_uint(vp[u][d]) & 0x7FFFFFFFu));
+      if (kDep && p + 32 * u < n) dep.add(frac_k(cell_frac(xp[u], jd, inv_dx)), order);
+    }
   }
-  if (!ok) return false;
+#pragma unroll
+  for (int d = 0; d < D; ++d) vmax[d] = warp_imax(vmax[d]);
+  return __all_sync(0xffffffffu, same);
+}
+
+// the 128-bit sums [sum d (D), sum d d^T (upper, NM)] of an equal-weight cell
+// (n particles, velocities v[d * ldv + p], shift = the first particle) in units
+// of 2^eq_d (2^(eq_x + eq_y) for the products), on the integer pipe,
+// lane-parallel over particles, by chunks of kSplitTerms a lane.  Lane l
+// returns sum warp_rs_index<kK1Sums<D>>(l).
+template <int D>
+constexpr int kK1Sums = D == 1 ? 4 : 16;
+template <int D>
+__device__ __forceinline__ __int128 fixed_sums(const float* __restrict__ v, int64_t ldv, int n, int lane,
+                                               const int (&eq)[D]) {
+  constexpr int NM = D * (D + 1) / 2;
   long long s0[D];
 #pragma unroll
   for (int d = 0; d < D; ++d) s0[d] = fixq(v[d * ldv], eq[d]);
+  __int128 tot = 0;
+  for (int c0 = 0; c0 < n; c0 += 32 * kSplitTerms) {
+    const int end = n - c0 < 32 * kSplitTerms ? n : c0 + 32 * kSplitTerms;
+    long long s1[D];
+    SplitSum s2[NM];
 #pragma unroll
-  for (int d = 0; d < D; ++d) s1[d] = 0;
+    for (int d = 0; d < D; ++d) s1[d] = 0;
+    for (int p = c0 + lane; p < end; p += 32 * kBatch) {
+      float vp[kBatch][D];
 #pragma unroll
-  for (int t = 0; t < NM; ++t) s2[t] = 0;
-#pragma unroll 2
-  for (int p = lane; p < n; p += 32) {
-    long long dq[D];
+      for (int u = 0; u < kBatch; ++u)
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-      dq[d] = fixq(v[d * ldv + p], eq[d]) - s0[d];
-      s1[d] += (__int128)dq[d];
+        for (int d = 0; d < D; ++d) vp[u][d] = v[d * ldv + min(p + 32 * u, end - 1)];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        if (p + 32 * u >= end) break;
+        SplitInt q[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+          const long long dq = fixq(vp[u][d], eq[d]) - s0[d];
+          s1[d] += dq;
+          q[d] = SplitInt(dq);
+        }
+        int t = 0;
+#pragma unroll
+        for (int i = 0; i < D; ++i)
+#pragma unroll
+          for (int k = i; k < D; ++k, ++t) {
+            if (k == i) s2[t].add_square(q[i]);
+            else s2[t].add(q[i], q[k]);
+          }
+      }
     }
+    __int128 w[kK1Sums<D>];
+#pragma unroll
+    for (int i = 0; i < kK1Sums<D>; ++i) w[i] = 0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) w[d] = s1[d];
     int t = 0;
 #pragma unroll
-    for (int x = 0; x < D; ++x)
+    for (int i = 0; i < D; ++i)
 #pragma unroll
-      for (int y = x; y < D; ++y, ++t) s2[t] += (__int128)dq[x] * (__int128)dq[y];
+      for (int k = i; k < D; ++k, ++t) w[D + t] = k == i ? s2[t].total_square() : s2[t].total();
+    tot += warp_rs_i128<kK1Sums<D>>(w, lane);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int d = 0; d < D; ++d) s1[d] += shfl_xor_i128(s1[d], o);
-#pragma unroll
-    for (int t = 0; t < NM; ++t) s2[t] += shfl_xor_i128(s2[t], o);
-  }
-  return true;
+  return tot;
 }
 
 // Per-cell record between the two kernels.  fixed = 1: the integer sums
@@ -177,8 +211,15 @@ struct K1Params {
 // go to the EM kernel's list; for the others the moment sums about the first
 // particle go to the cell's K1Raw record, and the parameter slots past the
 // first are cleared.
+//
+// Issue slots and the latency of the loads share the time.  1.5e8 equal-weight
+// 3V particles in 262144 cells: 2.98 ms with four passes a cell (weights,
+// deposit, exponents, sums) and 128-bit products; 2.38 with one scan and the
+// velocity sums from L1, batched loads and SplitSum products (4.2 GB, 0.62 ms
+// of traffic).  Four CTAs an SM: five (96 registers) took 2.42, six (80, with
+// spills) 2.74.
 template <int D, typename VT, int NW>
-__global__ void __launch_bounds__(NW * 32) em_k1_kernel(K1Params a) {
+__global__ void __launch_bounds__(NW * 32, 4) em_k1_kernel(K1Params a) {
   constexpr int NM = D * (D + 1) / 2;
   constexpr int NS = 1 + D + NM;
   constexpr int NP = NS <= 4 ? 4 : 16;
@@ -191,11 +232,36 @@ __global__ void __launch_bounds__(NW * 32) em_k1_kernel(K1Params a) {
     const int64_t off = a.cell_off[j];
     const int N = (int)(a.cell_off[j + 1] - off);
     const int K0 = a.init_K[j] < a.Kmax ? a.init_K[j] : a.Kmax;
-    // the weights' bit-for-bit equality, shared by the deposit and the sums
-    const bool same = N > 0 && N <= kFixMaxN && equal_weights(a.alpha, off, N, lane);
-    if (a.dep_rec) deposit_cell(j, off, N, a.x, a.alpha, a.inv_dx, a.order, a.dep_rec + (size_t)j * kDepWords,
-                                lane, same);
-    if (K0 != 1 && N > 0) {  // several (or no) supplied components: EM
+    const double* al = a.alpha + off;
+    const bool one = K0 == 1 && N > 0;  // else several (or no) supplied components, or an empty cell
+    long long* dep = a.dep_rec ? a.dep_rec + (size_t)j * kDepWords : nullptr;
+    // equal weights (bit for bit, positive), finite FP32 velocities and at most
+    // 2^14 particles: exact sums on the integer pipe
+    bool same = N > 0 && N <= kFixMaxN, fixed = false, dep_done = false;
+    int eq[D];
+    if (sizeof(VT) == 4 && same && one) {
+      const float* vf = reinterpret_cast<const float*>(vin) + off;
+      DepSums ds;
+      same = dep ? k1_scan<D, true>(al, vf, a.n, a.x + off, (double)j, a.inv_dx, a.order, N, lane, eq, ds)
+                 : k1_scan<D, false>(al, vf, a.n, nullptr, 0.0, 0.0, 0, N, lane, eq, ds);
+      const long long a0b = __double_as_longlong(al[0]);
+      if (dep && same) {
+        ds.put(a0b, N, a.order, dep, lane);
+        dep_done = true;
+      }
+      // a0 > 0 on the bits: positive sign, not a NaN
+      fixed = same && a0b > 0 && a0b <= 0x7FF0000000000000ll;
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        const int e = eq[d] >> 23;
+        fixed = fixed && e < 255;
+        eq[d] = (e ? e - 127 : -126) + 1 - kFixBits;
+      }
+    } else if (same) {
+      same = equal_weights(a.alpha, off, N, lane);
+    }
+    if (dep && !dep_done) deposit_cell(j, off, N, a.x, a.alpha, a.inv_dx, a.order, dep, lane, same);
+    if (!one && N > 0) {
       if (lane == 0) a.list[atomicAdd(a.list_count, 1u)] = (unsigned int)j;
       continue;
     }
@@ -205,35 +271,20 @@ __global__ void __launch_bounds__(NW * 32) em_k1_kernel(K1Params a) {
     for (int i = P + lane; i < a.Kmax * P; i += 32) prm_out[i] = 0.0;
     if (N == 0) continue;
     K1Raw<D>& r = raw[j];
-    bool fixed = false;
     if constexpr (sizeof(VT) == 4) {
-      // equal weights (bit for bit, positive) and at most 2^14 particles:
-      // exact sums on the integer pipe
-      if (same) {
-        const long long a0b = __double_as_longlong(a.alpha[off]);
-        // a0 > 0 on the bits: positive sign, not a NaN
-        if (a0b > 0 && a0b <= 0x7FF0000000000000ll) {
-          __int128 s1[D], s2[NM];
-          int eq[D];
-          fixed = fixed_sums<D>(reinterpret_cast<const float*>(vin) + off, a.n, N, lane, s1, s2, eq);
-          if (fixed) {
-            __int128 mine = 0;
+      if (fixed) {
+        const float* vf = reinterpret_cast<const float*>(vin) + off;
+        const __int128 tot = fixed_sums<D>(vf, a.n, N, lane, eq);
+        constexpr int NQ = kK1Sums<D>;
+        const int t = warp_rs_index<NQ>(lane);
+        if (t < D + NM && lane == warp_rs_lane<NQ>(t))  // the first of the lanes that hold the sum
+          *reinterpret_cast<longlong2*>(&r.w[2 * t]) =
+              make_longlong2((long long)(unsigned long long)tot, (long long)(tot >> 64));
+        if (lane == 0) {
+          r.a0 = al[0];
 #pragma unroll
-            for (int t = 0; t < D; ++t)
-              if (lane == t) mine = s1[t];
-#pragma unroll
-            for (int t = 0; t < NM; ++t)
-              if (lane == D + t) mine = s2[t];
-            if (lane < D + NM)
-              *reinterpret_cast<longlong2*>(&r.w[2 * lane]) =
-                  make_longlong2((long long)(unsigned long long)mine, (long long)(mine >> 64));
-            if (lane == 0) {
-              r.a0 = __longlong_as_double(a0b);
-#pragma unroll
-              for (int d = 0; d < D; ++d) r.eq[d] = eq[d];
-              r.fixed = 1;
-            }
-          }
+          for (int d = 0; d < D; ++d) r.eq[d] = eq[d];
+          r.fixed = 1;
         }
       }
     }

@@ -405,13 +405,6 @@ __device__ __forceinline__ void warp_rs(float (&v)[NP], int lane) {
 #pragma unroll
   for (int b = 16 >> LV; b >= 1; b >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], b);
 }
-template <int NP>
-__device__ __forceinline__ int warp_rs_index(int lane) {
-  int q = 0;
-#pragma unroll
-  for (int lv = 0; (NP >> lv) > 1; ++lv) q += ((lane >> (4 - lv)) & 1) * (NP >> (lv + 1));
-  return q;
-}
 
 // warp sums of NP doubles by recursive halving (the FP64 form of warp_rs):
 // lane l ends with the total of value warp_rs_index<NP>(l) in v[0]

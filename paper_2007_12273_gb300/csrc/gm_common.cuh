@@ -126,30 +126,27 @@ __device__ __forceinline__ double odd_2m53(unsigned long long k, bool neg) {
 constexpr int kFixBits = 54;
 constexpr int kFixMaxN = 1 << 14;
 
-// v / 2^eq rounded to the nearest integer (ties away from zero), from the
-// bit pattern of an FP32 v with |v| < 2^(eq + kFixBits)
+// v / 2^eq rounded to the nearest integer (ties away from zero), from the bit
+// pattern of v with |v| < 2^(eq + kBits): the significand at the top of the
+// range, shifted down by the value's distance from it (one shift for every
+// value; a shift either way by its sign was 10 instructions longer)
+template <int kBits = kFixBits>
 __device__ __forceinline__ long long fixq(float v, int eq) {
   const uint32_t u = __float_as_uint(v);
-  const int eb = (int)((u >> 23) & 0xFFu);
-  const long long m = (long long)((u & 0x7FFFFFu) | (eb ? 0x800000u : 0u));
-  const int sh = (eb ? eb - 150 : -149) - eq;  // v = m 2^(eb - 150) (subnormal: 2^-149)
-  long long r = 0;
-  if (sh >= 0) r = m << sh;
-  else if (sh > -40) r = (m + (1ll << (-sh - 1))) >> (-sh);
-  return (u >> 31) ? -r : r;
+  const int eb = (int)((u >> 23) & 0xFFu), e = eb > 0 ? eb : 1;  // v = m 2^(e - 150)
+  const unsigned long long m = (unsigned long long)((u & 0x7FFFFFu) | (eb ? 0x800000u : 0u)) << (kBits - 23);
+  const int down = min(eq + kBits + 126 - e, 63);  // 0 at the top
+  const long long r = (long long)(((m >> down) + 1ull) >> 1), s = (long long)((int)u >> 31);
+  return (r ^ s) - s;
 }
-
-// d / 2^eq rounded to the nearest integer (ties away from zero), from the
-// bit pattern of an FP64 d with |d| < 2^(eq + 62)
+template <int kBits = 62>
 __device__ __forceinline__ long long fixq(double d, int eq) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(d);
-  const int e = (int)((u >> 52) & 0x7FFull);
-  const long long m = (long long)((u & ((1ull << 52) - 1ull)) | (e ? (1ull << 52) : 0ull));
-  const int sh = (e ? e : 1) - 1075 - eq;  // d = m 2^(e - 1075)
-  long long r = 0;
-  if (sh >= 0) r = m << (sh < 9 ? sh : 9);
-  else if (sh > -60) r = (m + (1ll << (-sh - 1))) >> (-sh);
-  return (u >> 63) ? -r : r;
+  const int eb = (int)((u >> 52) & 0x7FFull), e = eb > 0 ? eb : 1;  // d = m 2^(e - 1075)
+  const unsigned long long m = ((u & ((1ull << 52) - 1ull)) | (eb ? (1ull << 52) : 0ull)) << (kBits - 52);
+  const int down = min(eq + kBits + 1022 - e, 63);
+  const long long r = (long long)(((m >> down) + 1ull) >> 1), s = (long long)u >> 63;
+  return (r ^ s) - s;
 }
 
 // Weighted sums in fixed point.  The weights and the velocities (or the
@@ -199,9 +196,7 @@ struct TermShift {
   __device__ __forceinline__ long long operator()(long long v) const { return (v + half) >> s; }
 };
 __device__ __forceinline__ int warp_imax(int v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+  return __reduce_max_sync(0xffffffffu, v);
 }
 
 __device__ __forceinline__ __int128 shfl_xor_i128(__int128 x, int b) {
@@ -210,18 +205,40 @@ __device__ __forceinline__ __int128 shfl_xor_i128(__int128 x, int b) {
   return ((__int128)hi << 64) | (__int128)(unsigned long long)lo;
 }
 
-// warp sums of NP 64-bit integers in 128 bits by recursive halving: lane l
-// ends with the total of value warp_rs_index<NP>(l)
+// value whose total lane l holds after a recursive halving of NP values
 template <int NP>
-__device__ __forceinline__ __int128 warp_rs_i128(const long long (&v)[NP], int lane) {
-  static_assert(NP == 4 || NP == 16, "4 or 16 values");
-  constexpr int LV = NP == 4 ? 2 : 4;
+__device__ __forceinline__ int warp_rs_index(int lane) {
+  int q = 0;
+#pragma unroll
+  for (int lv = 0; (NP >> lv) > 1; ++lv) q += ((lane >> (4 - lv)) & 1) * (NP >> (lv + 1));
+  return q;
+}
+// first lane holding the total of value q after a recursive halving of NP values
+template <int NP>
+__device__ __forceinline__ int warp_rs_lane(int q) {
+  int l = 0;
+#pragma unroll
+  for (int lv = 0; (NP >> lv) > 1; ++lv)
+    if (q & (NP >> (lv + 1))) l |= 16 >> lv;
+  return l;
+}
+
+// warp sums of NP integers (64 or 128 bits a lane) in 128 bits by recursive
+// halving: lane l ends with the total of value warp_rs_index<NP>(l)
+__device__ __forceinline__ __int128 shfl_xor_i128(long long x, int b) {
+  return (__int128)__shfl_xor_sync(0xffffffffu, x, b);
+}
+template <int NP, typename T>
+__device__ __forceinline__ __int128 warp_rs_i128(const T (&v)[NP], int lane) {
+  static_assert(NP == 4 || NP == 8 || NP == 16, "4, 8 or 16 values");
+  constexpr int LV = NP == 4 ? 2 : (NP == 8 ? 3 : 4);
   __int128 w[NP / 2];
   bool up = (lane & 16) != 0;
 #pragma unroll
-  for (int i = 0; i < NP / 2; ++i)
-    w[i] = (__int128)(up ? v[i + NP / 2] : v[i]) +
-           (__int128)__shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + NP / 2], 16);
+  for (int i = 0; i < NP / 2; ++i) {
+    const T send = up ? v[i] : v[i + NP / 2];
+    w[i] = (__int128)(up ? v[i + NP / 2] : v[i]) + shfl_xor_i128(send, 16);
+  }
 #pragma unroll
   for (int lv = 1; lv < LV; ++lv) {
     const int h2 = NP >> (lv + 1), b = 16 >> lv;
@@ -236,6 +253,39 @@ __device__ __forceinline__ __int128 warp_rs_i128(const long long (&v)[NP], int l
   for (int b = 16 >> LV; b >= 1; b >>= 1) w[0] += shfl_xor_i128(w[0], b);
   return w[0];
 }
+
+// Exact sums of products of integers below 2^55 on the 32 x 32-bit multiplier:
+// factors split as h 2^27 + l, and the sums of h h', h l' + l h' and l l' kept
+// apart in 64 bits each, up to kSplitTerms terms (squares of factors below
+// 0.96 x 2^54: 512), so that a term is a multiply-add per partial product (4
+// instructions, 3 for a square) instead of a 128-bit product and a 128-bit
+// addition (about 14).
+constexpr int kSplitTerms = 64;
+struct SplitInt {
+  int h, l;
+  __device__ __forceinline__ SplitInt() {}
+  __device__ __forceinline__ explicit SplitInt(long long v) : h((int)(v >> 27)), l((int)v & 0x7FFFFFF) {}
+};
+struct SplitSum {
+  long long hh = 0, hl = 0, ll = 0;
+  __device__ __forceinline__ void add(const SplitInt& a, const SplitInt& b) {
+    hh += (long long)a.h * b.h;
+    hl += (long long)a.h * b.l;
+    hl += (long long)a.l * b.h;
+    ll += (long long)a.l * b.l;
+  }
+  __device__ __forceinline__ void add_square(const SplitInt& a) {  // h l once: total_square
+    hh += (long long)a.h * a.h;
+    hl += (long long)a.h * a.l;
+    ll += (long long)a.l * a.l;
+  }
+  __device__ __forceinline__ __int128 total() const {
+    return ((__int128)hh << 54) + ((__int128)hl << 27) + (__int128)ll;
+  }
+  __device__ __forceinline__ __int128 total_square() const {
+    return ((__int128)hh << 54) + ((__int128)hl << 28) + (__int128)ll;
+  }
+};
 
 // a 128-bit integer times 2^e as the nearest-ish double (two roundings), from
 // its sign and magnitude: a small negative sum's low word as it stands is near

@@ -141,14 +141,11 @@ __global__ void __launch_bounds__(NW * 32) recon2d_stats_kernel(
     if (fix_plan<D>(rc, n, lane, eq, dzqs[wid])) {
       const bool several = rc.K > 1;
       long long sp[kPos2d], sf[D];
-      __int128 sq[D];
+      SplitSum sq[D];
 #pragma unroll
       for (int t = 0; t < kPos2d; ++t) sp[t] = 0;
 #pragma unroll
-      for (int d = 0; d < D; ++d) {
-        sf[d] = 0;
-        sq[d] = 0;
-      }
+      for (int d = 0; d < D; ++d) sf[d] = 0;
       for (int64_t i = lane; i < n; i += 32) {
         uint64_t m0;
         int z;
@@ -188,7 +185,7 @@ __global__ void __launch_bounds__(NW * 32) recon2d_stats_kernel(
           long long fq = fixq(f[d], eq[d]);
           if (several) fq += dzqs[wid][z][d];
           sf[d] += fq;
-          sq[d] += (__int128)fq * (__int128)fq;
+          sq[d].add_square(SplitInt(fq));
         }
       }
       __int128 sm[NS];
@@ -197,7 +194,7 @@ __global__ void __launch_bounds__(NW * 32) recon2d_stats_kernel(
 #pragma unroll
       for (int d = 0; d < D; ++d) {
         sm[kPos2d + d] = (__int128)sf[d];
-        sm[kPos2d + D + d] = sq[d];
+        sm[kPos2d + D + d] = sq[d].total_square();
       }
       put_fixed<D, kPos2d>(rw, sm, eq, lane);
     } else {

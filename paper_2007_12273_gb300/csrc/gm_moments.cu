@@ -81,7 +81,7 @@ __global__ void deposit_combine_kernel(int64_t C, const long long* rec, int orde
 // 2^kSlack times (its small terms would lose bits) sums in FP64 (13 operations
 // a particle for D = 3).  A CTA per cell with 28 FP64 operations a particle and
 // FP64 sums over its warps took 2.83 ms for 65536 3V cells of 572 weighted
-// particles (FP64 pipe); moments and deposit together went from 3.57 to 1.36 ms
+// particles (FP64 pipe); moments and deposit together went from 3.55 to 1.25 ms
 // (1.1 GB: issue slots bound both now).  Six CTAs an SM (80 registers) hide the
 // loads and the reductions better than five (95).  E = tr(M2) / 2.
 constexpr int kSlack = 4;
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_
             long long vq[D], av[D];
 #pragma unroll
             for (int d = 0; d < D; ++d) {
-              vq[d] = fixq(vj[(int64_t)d * n + q], qv[d]);
+              vq[d] = fixq<kScaleBits>(vj[(int64_t)d * n + q], qv[d]);
               av[d] = __mul64hi(a, vq[d]);  // below 2^60, units of 2^(qa + qv + 64)
               s[1 + d] += s1(av[d]);
             }

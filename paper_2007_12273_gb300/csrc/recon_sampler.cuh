@@ -410,17 +410,16 @@ __device__ __forceinline__ bool fix_plan(const RecCell<D>& rc, int64_t n, int la
 }
 // the warp's integer sums sm into cell record r
 template <int D, int NP>
-__device__ __forceinline__ void put_fixed(RecRaw<D, NP>& r, __int128 (&sm)[NP + 2 * D], const int (&eq)[D],
+__device__ __forceinline__ void put_fixed(RecRaw<D, NP>& r, const __int128 (&sm)[NP + 2 * D], const int (&eq)[D],
                                           int lane) {
-  __int128 mine = 0;
+  constexpr int NS = NP + 2 * D, NQ = NS <= 4 ? 4 : (NS <= 8 ? 8 : 16);
+  __int128 w[NQ];
 #pragma unroll
-  for (int t = 0; t < NP + 2 * D; ++t) {
-#pragma unroll
-    for (int o2 = 16; o2 > 0; o2 >>= 1) sm[t] += shfl_xor_i128(sm[t], o2);
-    if (lane == t) mine = sm[t];
-  }
-  if (lane < NP + 2 * D)
-    *reinterpret_cast<longlong2*>(&r.w[2 * lane]) =
+  for (int t = 0; t < NQ; ++t) w[t] = t < NS ? sm[t < NS ? t : 0] : (__int128)0;
+  const __int128 mine = warp_rs_i128<NQ>(w, lane);
+  const int t = warp_rs_index<NQ>(lane);
+  if (t < NS && lane == warp_rs_lane<NQ>(t))  // the first of the lanes that hold the sum
+    *reinterpret_cast<longlong2*>(&r.w[2 * t]) =
         make_longlong2((long long)(unsigned long long)mine, (long long)(mine >> 64));
   if (lane == 0) {
 #pragma unroll
