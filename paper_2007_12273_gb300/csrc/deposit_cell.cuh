@@ -110,19 +110,29 @@ __device__ __forceinline__ void deposit_cell(int64_t j, int64_t o, int64_t n, co
       const int eq = scale_exp(ea, 0.0);
       const TermShift sh(m, 62);
       long long s0 = 0, s1 = 0, s2 = 0;  // units of 2^(eq + sh.s)
-#pragma unroll 2
-      for (int p = lane; p < m; p += 32) {
-        const long long k = frac_k(cell_frac(x[c0 + p], jd, inv_dx));
-        const long long a = fixq(alpha ? alpha[c0 + p] : 1.0, eq), X = k << 11;  // s = X 2^-64
-        const long long as = __mul64hi(a, X);
-        s0 += sh(a);
-        if (order == 1) {
-          const long long t = sh(as);
-          s1 -= k < 0 ? t : 0;
-          s2 += k > 0 ? t : 0;
-        } else {
-          s1 += sh(as);
-          s2 += sh(__mul64hi(as, X));
+      for (int p0 = lane; p0 < m; p0 += 128) {  // the loads of four particles together
+        double xp[4], ap[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int p = min(p0 + 32 * u, m - 1);
+          xp[u] = x[c0 + p];
+          ap[u] = alpha ? alpha[c0 + p] : 1.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (p0 + 32 * u >= m) break;
+          const long long k = frac_k(cell_frac(xp[u], jd, inv_dx));
+          const long long a = fixq(ap[u], eq), X = k << 11;  // s = X 2^-64
+          const long long as = __mul64hi(a, X);
+          s0 += sh(a);
+          if (order == 1) {
+            const long long t = sh(as);
+            s1 -= k < 0 ? t : 0;
+            s2 += k > 0 ? t : 0;
+          } else {
+            s1 += sh(as);
+            s2 += sh(__mul64hi(as, X));
+          }
         }
       }
       __int128 t0 = s0, t1 = s1, t2 = s2;

@@ -81,10 +81,12 @@ __global__ void deposit_combine_kernel(int64_t C, const long long* rec, int orde
 // 2^kSlack times (its small terms would lose bits) sums in FP64 (13 operations
 // a particle for D = 3).  A CTA per cell with 28 FP64 operations a particle and
 // FP64 sums over its warps took 2.83 ms for 65536 3V cells of 572 weighted
-// particles (FP64 pipe); moments and deposit together went from 3.55 to 1.25 ms
-// (1.1 GB: issue slots bound both now).  Six CTAs an SM (80 registers) hide the
+// particles (FP64 pipe); moments and deposit together went from 3.55 to 1.16 ms
+// (1.1 GB; issue and the latency of the loads share it: one load in flight a
+// lane took 1.25).  Six CTAs an SM (80 registers) hide the
 // loads and the reductions better than five (95).  E = tr(M2) / 2.
 constexpr int kSlack = 4;
+constexpr int kLoads = 4;  // particles a lane whose loads are issued together
 template <int D, int NW, typename VT>
 __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_t C, int64_t n, const int64_t* cell_off,
                                                           const VT* v, const double* alpha, double* W,
@@ -136,22 +138,35 @@ __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_
         long long s[NP];
 #pragma unroll
         for (int t = 0; t < NP; ++t) s[t] = 0;
-        for (int q = lane; q < cnt; q += 32) {
-          const long long a = fixq(al[q], qa);
-          s[0] += s0(a);
-          if (vj) {
-            long long vq[D], av[D];
+        for (int q0 = lane; q0 < cnt; q0 += 32 * kLoads) {
+          double ap[kLoads];
+          VT vp[kLoads][D];
 #pragma unroll
-            for (int d = 0; d < D; ++d) {
-              vq[d] = fixq<kScaleBits>(vj[(int64_t)d * n + q], qv[d]);
-              av[d] = __mul64hi(a, vq[d]);  // below 2^60, units of 2^(qa + qv + 64)
-              s[1 + d] += s1(av[d]);
+          for (int u = 0; u < kLoads; ++u) {
+            const int q = min(q0 + 32 * u, cnt - 1);
+            ap[u] = al[q];
+#pragma unroll
+            for (int d = 0; d < D; ++d) vp[u][d] = vj ? vj[(int64_t)d * n + q] : VT(0);
+          }
+#pragma unroll
+          for (int u = 0; u < kLoads; ++u) {
+            if (q0 + 32 * u >= cnt) break;
+            const long long a = fixq(ap[u], qa);
+            s[0] += s0(a);
+            if (vj) {
+              long long vq[D], av[D];
+#pragma unroll
+              for (int d = 0; d < D; ++d) {
+                vq[d] = fixq<kScaleBits>(vp[u][d], qv[d]);
+                av[d] = __mul64hi(a, vq[d]);  // below 2^60, units of 2^(qa + qv + 64)
+                s[1 + d] += s1(av[d]);
+              }
+              int t = 1 + D;
+#pragma unroll
+              for (int x = 0; x < D; ++x)
+#pragma unroll
+                for (int y = x; y < D; ++y, ++t) s[t] += s1(__mul64hi(av[x] << 2, vq[y]));
             }
-            int t = 1 + D;
-#pragma unroll
-            for (int x = 0; x < D; ++x)
-#pragma unroll
-              for (int y = x; y < D; ++y, ++t) s[t] += s1(__mul64hi(av[x] << 2, vq[y]));
           }
         }
         const int i = warp_rs_index<NP>(lane);
