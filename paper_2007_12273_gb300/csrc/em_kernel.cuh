@@ -1521,8 +1521,9 @@ __device__ __forceinline__ void em_cell_body(const EmParams& a, uint32_t c_off, 
     // summed in FP64.  r_p goes over the tile's s_p and m_p arrays (8 bytes per
     // particle) and m_p over its terms; the weights stay for the last exact
     // pass.
-    // A thread takes the same groups' lanes in all passes below, so it reads
-    // back only what it wrote.  The component passes recompute
+    // The whole team shares this pass, so that a team of more warps than the
+    // cell has groups idles none; the groups' warps read other warps' particles
+    // after the barrier.  The component passes recompute
     // 2^(log2(u_k f_k) - m_p) with the same instructions on the same operands,
     // so sum_k gamma_pk = alpha_p N / W to FP64 rounding.
     double* Rd = reinterpret_cast<double*>(SMT);
@@ -1539,6 +1540,7 @@ __device__ __forceinline__ void em_cell_body(const EmParams& a, uint32_t c_off, 
       Rd[p] = a.alpha[off + p] * nw / Ssum;
       Mf[p] = m;
     }
+    TM.sync();
     for (int k = 0; k < K; ++k) {
       double ck[D];
 #pragma unroll
