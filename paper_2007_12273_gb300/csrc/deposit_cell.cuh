@@ -97,7 +97,9 @@ __device__ __forceinline__ void deposit_cell(int64_t j, int64_t o, int64_t n, co
     return;
   }
   // otherwise by chunks of kSumChunk particles: in fixed point (see
-  // kScaleBits), or in FP64 where a weight is not finite
+  // kScaleBits), or in FP64 where a weight is not finite or the weights spread
+  // too far (keeps_bits): the sum of the weights, to which the quadratic
+  // B-spline's parts add up, and for CIC each side's part, which stands alone
   ChunkSum tot;  // sum t on lane t < 3
   for (int64_t c0 = o; c0 < o + n; c0 += kSumChunk) {
     const int m = (int)(o + n - c0 < kSumChunk ? o + n - c0 : kSumChunk);
@@ -105,8 +107,9 @@ __device__ __forceinline__ void deposit_cell(int64_t j, int64_t o, int64_t n, co
 #pragma unroll 4
     for (int p = lane; p < m; p += 32) ea = max(ea, exp_field(alpha ? alpha[c0 + p] : 1.0));
     ea = warp_imax(ea);
+    bool fixed = exp_finite(ea, 0.0);
     double mine;
-    if (exp_finite(ea, 0.0)) {
+    if (fixed) {
       const int eq = scale_exp(ea, 0.0);
       const TermShift sh(m, 62);
       long long s0 = 0, s1 = 0, s2 = 0;  // units of 2^(eq + sh.s)
@@ -143,7 +146,10 @@ __device__ __forceinline__ void deposit_cell(int64_t j, int64_t o, int64_t n, co
         t2 += shfl_xor_i128(t2, q);
       }
       mine = i128_to_f64(lane == 0 ? t0 : (lane == 1 ? t1 : t2), eq + sh.s);
-    } else {
+      fixed = keeps_bits(t0, m, 62, sh) &&
+              (order != 1 || (keeps_bits(t1, m, 62, sh) && keeps_bits(t2, m, 62, sh)));
+    }
+    if (!fixed) {
       double a0 = 0.0, a1 = 0.0, a2 = 0.0;
       for (int p = lane; p < m; p += 32) {
         const double sx = cell_frac(x[c0 + p], jd, inv_dx) - 0.5;

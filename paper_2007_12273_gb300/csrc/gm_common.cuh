@@ -195,6 +195,18 @@ struct TermShift {
   }
   __device__ __forceinline__ long long operator()(long long v) const { return (v + half) >> s; }
 };
+// Whether a chunk's sum keeps the bits of its own terms.  Terms are rounded on
+// the scale of the largest product's bound: to a unit of 2^-kBits of it for
+// terms below 2^kBits, before their shift.  A sum whose m terms are
+// 2^-kSpread of the bound on average is then off by 2^-53 of itself or less; below
+// that (the large factors on different particles, or on those of another sum) the chunk
+// takes FP64 sums.  t: the sum of terms of one sign, or of magnitudes.  Uniform
+// weights and Gaussian velocities stand at 2^-3 to 2^-7.
+constexpr int kSpread = 8;
+__device__ __forceinline__ bool keeps_bits(__int128 t, int m, int bits, const TermShift& sh) {
+  const unsigned __int128 mag = t < 0 ? -(unsigned __int128)t : (unsigned __int128)t;
+  return (long long)(mag >> (bits - kSpread - sh.s)) >= m;
+}
 __device__ __forceinline__ int warp_imax(int v) {
   return __reduce_max_sync(0xffffffffu, v);
 }
