@@ -178,6 +178,14 @@ struct ChunkSum {
 // biased exponent, and the exponent eq of fixq for values up to it
 __device__ __forceinline__ int exp_field(double d) { return (int)((__double_as_longlong(d) >> 52) & 0x7FF); }
 __device__ __forceinline__ int exp_field(float f) { return (int)((__float_as_uint(f) >> 23) & 0xFFu); }
+// bits of |d| in the order of the magnitudes to an exponent, zero for zero only,
+// and the biased exponent of the largest
+__device__ __forceinline__ int top_bits(double d) {
+  return (__double2hiint(d) & 0x7FFFFFFF) | (__double2loint(d) != 0 ? 1 : 0);
+}
+__device__ __forceinline__ int top_bits(float f) { return (int)(__float_as_uint(f) & 0x7FFFFFFFu); }
+__device__ __forceinline__ int top_exp(int bits, double) { return bits >> 20; }
+__device__ __forceinline__ int top_exp(int bits, float) { return bits >> 23; }
 __device__ __forceinline__ int scale_exp(int emax, double) { return (emax ? emax : 1) - 1022 - kScaleBits; }
 __device__ __forceinline__ int scale_exp(int emax, float) { return (emax ? emax : 1) - 126 - kScaleBits; }
 __device__ __forceinline__ bool exp_finite(int emax, double) { return emax < 0x7FF; }
@@ -195,13 +203,13 @@ struct TermShift {
   }
   __device__ __forceinline__ long long operator()(long long v) const { return (v + half) >> s; }
 };
-// Whether a chunk's sum keeps the bits of its own terms.  Terms are rounded on
-// the scale of the largest product's bound: to a unit of 2^-kBits of it for
-// terms below 2^kBits, before their shift.  A sum whose m terms are
-// 2^-kSpread of the bound on average is then off by 2^-53 of itself or less; below
-// that (the large factors on different particles, or on those of another sum) the chunk
-// takes FP64 sums.  t: the sum of terms of one sign, or of magnitudes.  Uniform
-// weights and Gaussian velocities stand at 2^-3 to 2^-7.
+// Whether a chunk's sum keeps the bits of its own terms.  Terms below 2^bits are
+// rounded to units, before their shift.  A sum whose m terms are 2^-kSpread of
+// the bound on average is then off by 2^-55 of the terms' magnitudes with 572
+// particles and 2^-53 with 32, about what FP64 sums of one sign are off by
+// (2^-54 and 2^-55); below that (the large factors on different particles, or on those
+// of another sum) the chunk takes FP64 sums.  t: the sum of terms of one sign, or
+// of magnitudes.  Uniform weights and Gaussian velocities stand at 2^-3 to 2^-7.
 constexpr int kSpread = 8;
 __device__ __forceinline__ bool keeps_bits(__int128 t, int m, int bits, const TermShift& sh) {
   const unsigned __int128 mag = t < 0 ? -(unsigned __int128)t : (unsigned __int128)t;

@@ -76,16 +76,16 @@ __global__ void deposit_combine_kernel(int64_t C, const long long* rec, int orde
 // chunks of kSumChunk particles.  A chunk of finite particles takes fixed-point
 // sums (see kScaleBits): a pass for the largest exponents, then alpha, alpha v
 // and alpha v v^T on the integer pipe, converted to FP64 a sum per lane.  A
-// chunk whose largest weight and largest velocity belong to different particles
-// so far apart that the bound of alpha v or alpha v^2 exceeds the largest one
-// 2^kSlack times (its small terms would lose bits) sums in FP64 (13 operations
-// a particle for D = 3).  A CTA per cell with 28 FP64 operations a particle and
+// chunk in which one of them does not keep the bits of its own terms
+// (keeps_bits) sums in FP64 (13 operations a particle for D = 3): the weight
+// and the diagonal of alpha v v^T by their totals, an off-diagonal by the sum of
+// its terms' magnitudes (a light x-velocity may meet every heavy y-velocity);
+// alpha v follows from the diagonal, as |v| >= v^2 / max|v|.  A CTA per cell with 28 FP64 operations a particle and
 // FP64 sums over its warps took 2.83 ms for 65536 3V cells of 572 weighted
-// particles (FP64 pipe); moments and deposit together went from 3.55 to 1.16 ms
+// particles (FP64 pipe); moments and deposit together went from 3.55 to 1.09 ms
 // (1.1 GB; issue and the latency of the loads share it: one load in flight a
 // lane took 1.25).  Six CTAs an SM (80 registers) hide the
 // loads and the reductions better than five (95).  E = tr(M2) / 2.
-constexpr int kSlack = 4;
 constexpr int kLoads = 4;  // particles a lane whose loads are issued together
 template <int D, int NW, typename VT>
 __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_t C, int64_t n, const int64_t* cell_off,
@@ -103,29 +103,25 @@ __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_
       const double* al = alpha + c0;
       const VT* vj = v ? v + c0 : nullptr;  // no velocities: the weights' sum alone
       // the largest exponents
-      int ea = 0, ev[D], e1[D], e2[D];  // of alpha, v, alpha v, alpha v^2
+      int ea = 0, ev[D];
+      bool moves[D];  // whether any velocity is not zero
 #pragma unroll
-      for (int d = 0; d < D; ++d) ev[d] = e1[d] = e2[d] = 0;
+      for (int d = 0; d < D; ++d) ev[d] = 0;
 #pragma unroll 4
       for (int q = lane; q < cnt; q += 32) {
-        const int xa = exp_field(al[q]);
-        ea = max(ea, xa);
+        ea = max(ea, exp_field(al[q]));
         if (vj)
 #pragma unroll
-          for (int d = 0; d < D; ++d) {
-            const int xv = exp_field(vj[(int64_t)d * n + q]);
-            ev[d] = max(ev[d], xv);
-            e1[d] = max(e1[d], xa + xv);
-            e2[d] = max(e2[d], xa + 2 * xv);
-          }
+          for (int d = 0; d < D; ++d) ev[d] = max(ev[d], top_bits(vj[(int64_t)d * n + q]));
       }
       ea = warp_imax(ea);
       bool fixed = exp_finite(ea, 0.0);
 #pragma unroll
       for (int d = 0; d < D; ++d) {
         ev[d] = warp_imax(ev[d]);
-        fixed = fixed && exp_finite(ev[d], VT(0)) && ea + ev[d] - warp_imax(e1[d]) <= kSlack &&
-                ea + 2 * ev[d] - warp_imax(e2[d]) <= kSlack;
+        moves[d] = ev[d] != 0;
+        ev[d] = top_exp(ev[d], VT(0));
+        fixed = fixed && exp_finite(ev[d], VT(0));
       }
       double mine;
       if (fixed) {
@@ -136,8 +132,11 @@ __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_
         const TermShift s0(cnt, 62), s1(cnt, 60);
         // units: 2^(qa + s0.s); 2^(qa + qv + 64 + s1.s); 2^(qa + qv + qv' + 126 + s1.s)
         long long s[NP];
+        int mag[D == 3 ? 3 : 1];  // the off-diagonal terms' magnitudes, high words (below 2^30)
 #pragma unroll
         for (int t = 0; t < NP; ++t) s[t] = 0;
+#pragma unroll
+        for (int t = 0; t < (D == 3 ? 3 : 1); ++t) mag[t] = 0;
         for (int q0 = lane; q0 < cnt; q0 += 32 * kLoads) {
           double ap[kLoads];
           VT vp[kLoads][D];
@@ -165,7 +164,11 @@ __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_
 #pragma unroll
               for (int x = 0; x < D; ++x)
 #pragma unroll
-                for (int y = x; y < D; ++y, ++t) s[t] += s1(__mul64hi(av[x] << 2, vq[y]));
+                for (int y = x; y < D; ++y, ++t) {
+                  const long long w = s1(__mul64hi(av[x] << 2, vq[y]));
+                  s[t] += w;
+                  if (y > x) mag[x + y - 1] += abs((int)(w >> 32));
+                }
             }
           }
         }
@@ -177,8 +180,25 @@ __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_
         for (int x = 0; x < D; ++x)
 #pragma unroll
           for (int y = x; y < D; ++y, ++t) unit = i == t ? qa + qv[x] + qv[y] + 126 + s1.s : unit;
-        mine = i128_to_f64(warp_rs_i128<NP>(s, lane), unit);
-      } else {
+        const __int128 sum = warp_rs_i128<NP>(s, lane);
+        mine = i128_to_f64(sum, unit);
+        bool kept = i != 0 || keeps_bits(sum, cnt, 62, s0);
+#pragma unroll
+        for (int x = 0, t = 1 + D; x < D; t += D - x, ++x)
+          kept = kept && (i != t || !moves[x] || keeps_bits(sum, cnt, 60, s1));
+        fixed = __all_sync(0xffffffffu, kept);
+        if (D == 3) {
+#pragma unroll
+          for (int x = 0; x < D; ++x)
+#pragma unroll
+            for (int y = x + 1; y < D; ++y) {
+              const int q = x + y - 1;
+              const long long m = (long long)__reduce_add_sync(0xffffffffu, mag[q] >> 5) << 37;
+              fixed = fixed && (!moves[x] || !moves[y] || keeps_bits(m, cnt, 60, s1));
+            }
+        }
+      }
+      if (!fixed) {
         double acc[NP];
 #pragma unroll
         for (int i = 0; i < NP; ++i) acc[i] = 0.0;
