@@ -86,6 +86,11 @@ __global__ void deposit_combine_kernel(int64_t C, const long long* rec, int orde
 // (1.1 GB; issue and the latency of the loads share it: one load in flight a
 // lane took 1.25).  Six CTAs an SM (80 registers) hide the
 // loads and the reductions better than five (95).  E = tr(M2) / 2.
+// A cell of more than kBigCell particles is left to a whole CTA, after the
+// others: its chunks go round the CTA's warps, whose sums are added in their
+// order.  With a warp for every cell 152 3V cells of 1e5 particles took 3.66 ms
+// and one of 1e7 338; now 2.13 and 199, 1.8 and 170 of it the deposit.
+constexpr int kBigCell = 2 * kSumChunk;
 constexpr int kLoads = 4;  // particles a lane whose loads are issued together
 template <int D, int NW, typename VT>
 __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_t C, int64_t n, const int64_t* cell_off,
@@ -94,11 +99,28 @@ __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_
   constexpr int NM = D * (D + 1) / 2;
   constexpr int NS = 1 + D + NM;
   constexpr int NP = NS <= 4 ? 4 : 16;
+  __shared__ double parts[NW][NS][2];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int64_t j = (int64_t)blockIdx.x * NW + wid; j < C; j += (int64_t)gridDim.x * NW) {
-    const int64_t o = cell_off[j], end = cell_off[j + 1];
+  bool big = false;  // the second turn, for the CTA's big cells
+  int64_t j = (int64_t)blockIdx.x * NW + wid;
+  for (;;) {
+    if (j >= C) {
+      if (big) break;
+      // every warp gets here once, and they take the second turn together
+      bool any = false;
+      for (int64_t q = blockIdx.x + threadIdx.x * (int64_t)gridDim.x; q < C; q += NW * 32 * (int64_t)gridDim.x)
+        any = any || cell_off[q + 1] - cell_off[q] > kBigCell;
+      if (!__syncthreads_or(any)) break;
+      big = true;
+      j = blockIdx.x;
+      if (j >= C) break;
+    }
+    const int64_t jc = j, o = cell_off[jc], end = cell_off[jc + 1];
+    j += (int64_t)gridDim.x * (big ? 1 : NW);
+    if ((end - o > kBigCell) != big) continue;
+    const int64_t first = big ? o + (int64_t)wid * kSumChunk : o;
     ChunkSum tot;  // sum t on lane t < NS
-    for (int64_t c0 = o; c0 < end; c0 += kSumChunk) {
+    for (int64_t c0 = first; c0 < end; c0 += (big ? NW : 1) * kSumChunk) {
       const int cnt = (int)(end - c0 < kSumChunk ? end - c0 : kSumChunk);
       const double* al = alpha + c0;
       const VT* vj = v ? v + c0 : nullptr;  // no velocities: the weights' sum alone
@@ -223,17 +245,31 @@ __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_
         mine = acc[0];
       }
       mine = __shfl_sync(0xffffffffu, mine, warp_rs_lane<NP>(lane & (NP - 1)));
-      tot.add(mine, c0 == o);
+      tot.add(mine, c0 == first);
+    }
+    if (big) {
+      if (lane < NS) {
+        parts[wid][lane][0] = tot.s;
+        parts[wid][lane][1] = tot.e;
+      }
+      __syncthreads();
+      if (wid == 0 && lane < NS)
+        for (int w = 1; w < NW; ++w) {
+          tot.add(parts[w][lane][0], false);
+          tot.e += parts[w][lane][1];
+        }
+      __syncthreads();
+      if (wid != 0) continue;
     }
     const double mine = tot.value();
-    if (W && lane == 0) W[j] = mine;
-    if (p && lane >= 1 && lane <= D) p[j * D + lane - 1] = mine;
-    if (M2 && lane > D && lane < NS) M2[j * NM + lane - 1 - D] = mine;
+    if (W && lane == 0) W[jc] = mine;
+    if (p && lane >= 1 && lane <= D) p[jc * D + lane - 1] = mine;
+    if (M2 && lane > D && lane < NS) M2[jc * NM + lane - 1 - D] = mine;
     if (E) {
       double tr = __shfl_sync(0xffffffffu, mine, 1 + D);
       if (D == 3)
         tr = (tr + __shfl_sync(0xffffffffu, mine, 7 < NS ? 7 : 0)) + __shfl_sync(0xffffffffu, mine, 9 < NS ? 9 : 0);
-      if (lane == 0) E[j] = 0.5 * tr;
+      if (lane == 0) E[jc] = 0.5 * tr;
     }
   }
 }
@@ -302,7 +338,8 @@ cudaError_t launch_moments(int D, int64_t C, int64_t n, const int64_t* cell_off,
                            double* E, cudaStream_t s) {
   if (C == 0) return cudaSuccess;
   constexpr int NW = 4;
-  const int g = grid_for((C + NW - 1) / NW, 152 * 16);
+  // a CTA per cell as long as that leaves no more than a few on an SM
+  const int g = C <= 152 * 4 ? (int)C : grid_for((C + NW - 1) / NW, 152 * 16);
   if (D == 1) {
     if (v_f64)
       moments_kernel<1, NW, double><<<g, NW * 32, 0, s>>>(C, n, cell_off, (const double*)v, alpha, W, p, M2, E);
