@@ -75,7 +75,8 @@ struct EmParams {
   int team;      // threads of a team (a power of two, 32 .. 256)
   int nvw;       // partial sums per cell (2, 4 or 8 groups of 32 lanes, see Team)
   int granules;  // shared-memory pool, in units of kPoolGranule bytes
-  int patience;  // tries for a tile before the cell takes the global one
+  int share;     // a team's share of the pool
+  int patience;  // tries for a tile of up to a share before the cell takes the global one
   double tol;
   uint64_t seed;
 };
@@ -1839,8 +1840,15 @@ __global__ void __launch_bounds__(kEmThreads, 1) em_kernel(EmParams a) {
       const int Np = N + (N & 1);
       c.gn = (int)((em_tile_bytes(D, Np, c.eq != 0) + kPoolGranule - 1) / kPoolGranule);
       c.g0 = -1;
-      if (Np <= a.cap && c.gn <= a.granules)
-        for (int it = 0; it < a.patience && (c.g0 = pool_take(pool, a.granules, c.gn)) < 0; ++it) __nanosleep(2000);
+      // A cell within its team's share waits for a hole (the others' cells are
+      // of its kind, and free one in a few ms at most); a larger one takes what
+      // is free now or works in L2, where it would otherwise wait for the
+      // other teams' whole fits.
+      if (Np <= a.cap && c.gn <= a.granules) {
+        const int tries = c.gn <= a.share ? a.patience : 1;
+        for (int it = 0; it < tries && (c.g0 = pool_take(pool, a.granules, c.gn)) < 0; ++it)
+          if (it + 1 < tries) __nanosleep(2000);
+      }
     }
     TM.sync();
     if (tid == 0) {
