@@ -550,23 +550,24 @@ int gm_graph_destroy(gm_graph* g);
  * has no counterpart (it runs one cell per process on CPUs).
  *
  * Times gm_compress on a sample of the batch (the first 128 x #SM cells,
- * many per CTA) for every candidate shape: threads_per_cell in
- * {64, 128, 256} and shared-tile capacities smem_particles covering the
- * library default and the 90th, 99th, 100th and 50th percentiles of the
- * cell sizes (only those that fit in shared memory; larger cells use the
- * L2-resident global tile; small CTAs with small tiles put more cells on
- * an SM at once, which pays where per-cell serial phases dominate).  Each trial runs a fixed number of sweeps (tol = 0, max_sweeps =
+ * many per SM) for every candidate shape: threads_per_cell in
+ * {64, 128, 256} and shared-tile limits smem_particles: the library default
+ * (10240 in 1V, 7312 in 3V) and the 90th, 99th and 50th percentiles of the
+ * cell sizes where they lie below the largest (cells above the limit use the
+ * L2-resident global tile and leave the shared memory to the others).  Each
+ * trial runs a fixed number of sweeps (tol = 0, max_sweeps =
  * sweeps_per_trial, 0 = 24) so that every candidate does the same work,
  * and the fastest of two repetitions counts; the library default (256
  * threads, default tile) is kept unless another candidate is more than 3 %
- * faster.  Writes the winner into
+ * faster, and the default tile unless another one is for the same
+ * threads_per_cell.  Writes the winner into
  * cfg->threads_per_cell and cfg->smem_particles and, if timings_ms is not
  * NULL, the trial times (host array of at least GM_TUNE_CANDIDATES floats,
  * -1 for skipped candidates; candidate i has threads_per_cell
  * {64, 128, 256}[i % 3] and tile i / 3).
  * Arguments as gm_compress (device arrays); cell_off is copied to the host,
  * so the call synchronises `stream`.  Results of later gm_compress calls do
- * not depend on the tile; the CTA size changes the order of FP32 partial
+ * not depend on the tile; threads_per_cell changes the order of FP32 partial
  * sums only.  Returns GM_OK or an error code; cfg is unchanged on error.
  */
 #define GM_TUNE_CANDIDATES 15

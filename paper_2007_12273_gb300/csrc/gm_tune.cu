@@ -29,7 +29,7 @@ struct TrialOut {
 
 size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// candidates: CTA sizes x shared tiles; candidate i = (kTuneNT[i % 3], tile i / 3)
+// candidates: lanes of a cell's sums x shared tiles; candidate i = (kTuneNT[i % 3], tile i / 3)
 constexpr int kTuneThreads = 3;
 constexpr int kTuneNT[kTuneThreads] = {64, 128, 256};
 constexpr int kTuneCaps = 5;
@@ -57,8 +57,7 @@ int tune_impl(gm_config* cfg, int64_t C, int64_t n_particles, const int64_t* cel
   if (sms < 1) sms = 1;
 
   // cell sizes of the sample: the first 128 cells per SM (many cells per
-  // CTA even for the smallest CTAs, so that a trial measures throughput,
-  // not one wave)
+  // team, so that a trial measures throughput, not one wave)
   const int64_t S = std::min<int64_t>(C, (int64_t)128 * sms);
   std::vector<int64_t> off((size_t)S + 1);
   e = cudaMemcpyAsync(off.data(), cell_off, sizeof(int64_t) * (size_t)(S + 1), cudaMemcpyDeviceToHost, s);
@@ -72,7 +71,11 @@ int tune_impl(gm_config* cfg, int64_t C, int64_t n_particles, const int64_t* cel
     return sizes[i];
   };
 
-  // candidate shared tiles (particles, multiple of 4, within 200 KB)
+  // candidate shared tiles (particles, multiple of 4, within 200 KB).  The
+  // library's default is the largest one: every cell that fits the pool may have
+  // a shared tile.  A smaller limit sends the cells above it to L2 and leaves
+  // the pool to the others; a limit that no cell of the sample reaches is the
+  // default again.
   const int64_t max_cap = (int64_t)(200 * 1024) / ((int64_t)(D + 4) * 4) & ~(int64_t)3;
   std::vector<int> caps;
   auto add_cap = [&](int64_t c) {
@@ -81,11 +84,9 @@ int tune_impl(gm_config* cfg, int64_t C, int64_t n_particles, const int64_t* cel
     if (c > max_cap) return;
     if (std::find(caps.begin(), caps.end(), (int)c) == caps.end()) caps.push_back((int)c);
   };
-  add_cap(D == 1 ? 2559 : 3071);  // the library default
-  add_cap(quant(0.90));
-  add_cap(quant(0.99));
-  add_cap(sizes.back());
-  add_cap(quant(0.50));  // small tiles: more (smaller) CTAs per SM
+  add_cap(max_cap - 1);  // the library default
+  for (const double q : {0.90, 0.99, 0.50})
+    if (quant(q) < sizes.back()) add_cap(quant(q));
   if (caps.size() > (size_t)kTuneCaps) caps.resize(kTuneCaps);
 
   // trial outputs
@@ -160,13 +161,17 @@ int tune_impl(gm_config* cfg, int64_t C, int64_t n_particles, const int64_t* cel
   cudaEventDestroy(t1);
   cudaFree(o.base);
   if (rc != GM_OK) return rc;
-  // the library default (256 threads, default tile: candidate 2) stays
-  // unless another shape is faster by more than 3 %: trials closer than
-  // that are within the run-to-run spread
-  const int dflt = 2;
-  for (int i = 0; i < kTuneCands; ++i)
-    if (times[i] >= 0.0f && (best < 0 || times[i] < times[best])) best = i;
-  if (best >= 0 && times[dflt] >= 0.0f && times[best] > 0.97f * times[dflt]) best = dflt;
+  // the library default (256 lanes, default tile: candidate 2) stays unless
+  // another shape is faster by more than 3 %, and each number of lanes keeps
+  // the default tile (candidates 0 to 2) unless another is by as much: trials closer
+  // than that are within the run-to-run spread
+  for (int ti = kTuneThreads - 1; ti >= 0; --ti) {
+    int c = -1;
+    for (int i = ti; i < kTuneCands; i += kTuneThreads)
+      if (times[i] >= 0.0f && (c < 0 || times[i] < (c == ti ? 0.97f : 1.0f) * times[c])) c = i;
+    if (c >= 0 && (best < 0 || times[c] < (best % kTuneThreads == kTuneThreads - 1 ? 0.97f : 1.0f) * times[best]))
+      best = c;
+  }
   if (best < 0) return tune_fail(GM_ERR_CUDA, "no candidate ran");
   if (timings_ms)
     for (int i = 0; i < kTuneCands; ++i) timings_ms[i] = times[i];
