@@ -311,13 +311,16 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(const __grid_constant__ CU
 
 // ring depth: two stages (48 KB each for 128 x 256 tiles), so that two CTAs
 // share an SM (2 x 97 KB of shared memory, at most 2 x 256 TMEM columns)
-// and one's ring fill and epilogue overlap the other's MMAs.  The narrow
-// tiles run with few CTAs (below), where a CTA's own ring has to cover the
-// load latency: six stages of 20 KB, four of 24 KB.
-template <int BN>
-constexpr int gemm_stages() { return BN == 32 ? 6 : (BN == 64 ? 4 : 2); }
-template <int BN>
-constexpr size_t gemm_smem() { return (size_t)(kBM + BN) * kBK * 2 * gemm_stages<BN>() + 1024; }
+// and one's ring fill and epilogue overlap the other's MMAs.  Narrow tiles
+// take deeper rings: four stages of 20 or 24 KB, still two CTAs an SM; with no
+// more tiles than SMs (a training batch's weight gradients) a CTA's own ring
+// has to cover the load latency, and 32-column tiles take six, one CTA an SM.
+// 262144 x 32 x 256 (2048 tiles): 0.069 ms with six stages, 0.049 with four,
+// 0.052 with two; 16384 x 32 x 4096 (128 tiles) 0.042 with six.
+template <int BN, bool kAlone>
+constexpr int gemm_stages() { return BN == 32 ? (kAlone ? 6 : 4) : (BN == 64 ? 4 : 2); }
+template <int BN, bool kAlone>
+constexpr size_t gemm_smem() { return (size_t)(kBM + BN) * kBK * 2 * gemm_stages<BN, kAlone>() + 1024; }
 
 namespace {
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -365,12 +368,14 @@ cudaError_t launch_tc_gemm(const void* A, const void* A2, const void* B, int M, 
       !make_map(&mapB, B, N, K, ldb, bn))
     return cudaErrorInvalidValue;
   dim3 grid((unsigned)mt, (N + bn - 1) / bn);
-#define GM_TC_LAUNCH(BNV, TWO)                                                                   \
+  const bool alone = mt * ((N + bn - 1) / bn) <= 152;
+#define GM_TC_LAUNCH(BNV, ALONE, TWO)                                                            \
   {                                                                                              \
-    auto k = tc_gemm_kernel<BNV, gemm_stages<BNV>(), TWO>;                                        \
+    auto k = tc_gemm_kernel<BNV, gemm_stages<BNV, ALONE>(), TWO>;                                 \
     /* at least 80 KB of shared memory per CTA keeps two CTAs (2 x 256 TMEM columns) per SM at    \
        most, so a TMEM allocation never waits */                                                 \
-    const size_t smem = gemm_smem<BNV>() < 80 * 1024 ? 80 * 1024 : gemm_smem<BNV>();             \
+    constexpr size_t need = gemm_smem<BNV, ALONE>();                                             \
+    const size_t smem = need < 80 * 1024 ? 80 * 1024 : need;                                     \
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
                                          (int)smem);                                             \
     if (e != cudaSuccess) return e;                                                              \
@@ -378,14 +383,16 @@ cudaError_t launch_tc_gemm(const void* A, const void* A2, const void* B, int M, 
                               ldm, Cf, (__nv_bfloat16*)Cb, ldc, err);                             \
   }
   if (A2) {
-    if (bn == 32) GM_TC_LAUNCH(32, true)
-    else if (bn == 64) GM_TC_LAUNCH(64, true)
-    else GM_TC_LAUNCH(128, true)
+    if (bn == 32 && alone) GM_TC_LAUNCH(32, true, true)
+    else if (bn == 32) GM_TC_LAUNCH(32, false, true)
+    else if (bn == 64) GM_TC_LAUNCH(64, false, true)
+    else GM_TC_LAUNCH(128, false, true)
   } else {
-    if (bn == 32) GM_TC_LAUNCH(32, false)
-    else if (bn == 64) GM_TC_LAUNCH(64, false)
-    else if (bn == 128) GM_TC_LAUNCH(128, false)
-    else GM_TC_LAUNCH(256, false)
+    if (bn == 32 && alone) GM_TC_LAUNCH(32, true, false)
+    else if (bn == 32) GM_TC_LAUNCH(32, false, false)
+    else if (bn == 64) GM_TC_LAUNCH(64, false, false)
+    else if (bn == 128) GM_TC_LAUNCH(128, false, false)
+    else GM_TC_LAUNCH(256, false, false)
   }
 #undef GM_TC_LAUNCH
   return cudaGetLastError();
