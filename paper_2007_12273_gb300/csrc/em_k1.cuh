@@ -217,9 +217,14 @@ struct K1Params {
 // deposit, exponents, sums) and 128-bit products; 2.38 with one scan and the
 // velocity sums from L1, batched loads and SplitSum products (4.2 GB, 0.62 ms
 // of traffic).  Four CTAs an SM: five (96 registers) took 2.42, six (80, with
-// spills) 2.74.
+// spills) 2.74.  FP64 velocities have no scan and no batches: eight CTAs in 3V (64
+// registers) and ten in 1V (48), against six and seven (86 and 71 registers) 2.4e7
+// equal-weight particles in cells of 64 1.59 -> 1.55 and 0.81 -> 0.75 ms, of 4000
+// 0.95 -> 0.91 and 0.48 -> 0.42.
+template <int D, typename VT>
+constexpr int k1_ctas() { return sizeof(VT) == 4 ? 4 : (D == 3 ? 8 : 10); }
 template <int D, typename VT, int NW>
-__global__ void __launch_bounds__(NW * 32, 4) em_k1_kernel(K1Params a) {
+__global__ void __launch_bounds__(NW * 32, k1_ctas<D, VT>()) em_k1_kernel(K1Params a) {
   constexpr int NM = D * (D + 1) / 2;
   constexpr int NS = 1 + D + NM;
   constexpr int NP = NS <= 4 ? 4 : 16;
