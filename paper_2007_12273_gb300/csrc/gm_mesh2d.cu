@@ -418,7 +418,7 @@ __device__ __forceinline__ double mm2d_row(const Mesh2dSolve& m, int64_t i) {
 constexpr int kSolveThreads = 64;
 __global__ void __launch_bounds__(kSolveThreads) mm2d_solve_kernel(Mesh2dSolve m, CircTaps tx, CircTaps ty,
                                                                   int max_iter, int* converged) {
-  __shared__ double red[kSolveThreads / 32];
+  __shared__ unsigned long long red[kSolveThreads / 32];
   const double thr = m.tol * __longlong_as_double((long long)*m.scale);
   const int64_t C = m.Cx * m.Cy, step = (int64_t)gridDim.x * kSolveThreads;
   const int64_t i0 = blockIdx.x * (int64_t)kSolveThreads + threadIdx.x;
@@ -426,21 +426,23 @@ __global__ void __launch_bounds__(kSolveThreads) mm2d_solve_kernel(Mesh2dSolve m
   int conv = 0;
   for (int it = 0;; ++it) {
     // r_i = b_i - (M dA)_i on the rows of cells with particles (empty rows 0)
-    double mx = 0.0;
+    // (the largest |r| by its bits, in which NaN lies above infinity)
+    unsigned long long mx = 0ull;
     for (int64_t i = i0; i < C; i += step) {
       const double ri = out_count(m.out_off, i, m.n_out) > 0 ? m.b[i] - m.q * mm2d_row(m, i) : 0.0;
       m.r[i] = ri;
-      mx = fmax(mx, fabs(ri));
+      mx = max(mx, pos_bits(fabs(ri)));
     }
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
     __syncthreads();
     if (threadIdx.x == 0) {
-      for (int q = 1; q < kSolveThreads / 32; ++q) mx = fmax(mx, red[q]);
-      atomicMax(m.norm + it, pos_bits(mx));
+      for (int q = 1; q < kSolveThreads / 32; ++q) mx = max(mx, red[q]);
+      atomicMax(m.norm + it, mx);
     }
     if (!grid_barrier(m.arrived, phase++)) break;
-    conv = __longlong_as_double((long long)__ldcg(m.norm + it)) <= thr;
+    const double norm = __longlong_as_double((long long)__ldcg(m.norm + it));
+    conv = isfinite(norm) && norm <= thr;
     if (conv || it == max_iter) break;
     // t = (Tx^-1 along every row) r
     for (int64_t i = i0; i < C; i += step) {
