@@ -819,13 +819,18 @@ __device__ __noinline__ void exact_pass(uint32_t c_off, Team T, bool stats0, boo
   run_groups<D, R, kGlobal>(x, ExactStep<D, R, kGlobal>{x.c->K, x.c->c0, stats0, fresh});
 }
 template <int D, typename R, bool kGlobal, bool withL>
-__device__ __noinline__ void comp_pass(uint32_t c_off, Team T, int k) {
+__device__ __forceinline__ void comp_pass_here(uint32_t c_off, const Team& T, int k) {
   const PassCtx<D, R, kGlobal> x = pass_ctx<D, R, kGlobal>(c_off, T);
   const int ps = x.c->pstate;
   const float c0 = withL ? x.c->c0 : 0.0f;
   if (ps == 1) run_groups<D, R, kGlobal>(x, CompStep<D, R, kGlobal, withL, true>{k, ps, c0});
   else
   run_groups<D, R, kGlobal>(x, CompStep<D, R, kGlobal, withL, false>{k, ps, c0});
+}
+
+template <int D, typename R, bool kGlobal, bool withL>
+__device__ __noinline__ void comp_pass(uint32_t c_off, Team T, int k) {
+  comp_pass_here<D, R, kGlobal, withL>(c_off, T, k);
 }
 
 // Annihilation of component k (one thread): compaction, eq. (omegak)'s
@@ -1499,7 +1504,10 @@ __device__ __forceinline__ void em_cell_body(const EmParams& a, uint32_t c_off, 
     if (c.done) break;
     while (c.k < c.K) {
       const int k = c.k;
-      comp_pass<D, R, kGlobal, false>(c_off, TM, k);
+      // (in place beside the FP32 M-step: a call and its return take 260 cycles,
+      // 2 to 5 % of a fit; with the FP64 one the 3V kernel spills more than that)
+      if constexpr (sizeof(R) == 4 && !kGlobal) comp_pass_here<D, R, kGlobal, false>(c_off, TM, k);
+      else comp_pass<D, R, kGlobal, false>(c_off, TM, k);
       if (tid < 32) {
         if constexpr (sizeof(R) == 8) {
           mstep64<D, R>(c_off, k, TM, false);

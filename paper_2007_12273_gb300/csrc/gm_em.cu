@@ -13,6 +13,11 @@ namespace gmcr {
 //     64 registers 109, -; one CTA of 256 threads per cell (two or four per
 //     SM, the same work) 113, 284.
 //   * Smaller cells have only 1 to 4 groups of pairs: 2 warps, up to 10 teams.
+//     So do cells with the FP32 M-step, a tenth of the FP64 one, where at least 8
+//     tiles fit and more than 5 cells wait: the passes' latency is what is left
+//     to hide (4096 cells of 785, 24 sweeps: 1V 3.75 -> 3.15 ms, 3V 8.2 -> 8.1; 300
+//     particles 2.80 -> 2.13, 5.2 -> 4.3; 1216 cells of 785 1.31 -> 0.98, 2.88 -> 2.21;
+//     with 4 cells per SM two warps take 1.12 times as long).
 //   * No more teams than tiles of the mean size fit the pool (but two: a
 //     team without a tile works in L2, at once if the tile is larger than its
 //     share; 888 3V cells of 4500 particles 11.5 -> 8.8 ms against waiting for
@@ -27,8 +32,9 @@ cudaError_t launch_em(int D, int fp64_mstep, EmParams p, int sms, cudaStream_t s
   const int64_t mean = (p.n + p.C - 1) / p.C;
   const int64_t per_sm = (p.C + sms - 1) / sms;
   EmShape sh;
-  sh.team = mean > 256 ? 128 : 64;
-  const int64_t each = ctl + sh.team / 32 * em_buf_bytes(D) + em_tile_bytes(D, mean, true);
+  const int64_t each2 = ctl + 2 * em_buf_bytes(D) + em_tile_bytes(D, mean, true);  // with 2 warps
+  sh.team = mean > 256 && (fp64_mstep || per_sm <= 5 || kSmem / each2 < 8) ? 128 : 64;
+  const int64_t each = each2 + (sh.team / 32 - 2) * em_buf_bytes(D);
   int64_t T = kSmem / each;
   if (T < 2) T = 2;
   if (T > kEmThreads / sh.team) T = kEmThreads / sh.team;
