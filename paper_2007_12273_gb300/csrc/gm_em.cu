@@ -47,7 +47,14 @@ cudaError_t launch_em(int D, int fp64_mstep, EmParams p, int sms, cudaStream_t s
   p.patience = 1 << 15;  // 2 us each: a cell's fit takes a few ms
   p.granules = (int)((kSmem - 64 - T * ctl - T * sh.team / 32 * em_buf_bytes(D)) / kPoolGranule);
   if (p.granules > 32 * kPoolWords) p.granules = 32 * kPoolWords;
-  p.share = p.granules / (int)T;
+  // a team's share; where the others' tiles, at twice the mean, leave room for
+  // more, up to half of the pool (16384 log-normal 3V cells of 572: a cell of
+  // three times the mean waits for a hole rather than work in L2)
+  const int64_t mean_gn = (em_tile_bytes(D, mean, true) + kPoolGranule - 1) / kPoolGranule;
+  int64_t share = p.granules - 2 * (T - 1) * mean_gn;
+  if (share > p.granules / 2) share = p.granules / 2;
+  if (share < p.granules / T) share = p.granules / T;
+  p.share = (int)share;
   if (D == 1)
     return fp64_mstep ? em_go<1, double>(p, sh, kSmem, s) : em_go<1, float>(p, sh, kSmem, s);
   return fp64_mstep ? em_go<3, double>(p, sh, kSmem, s) : em_go<3, float>(p, sh, kSmem, s);
