@@ -14,10 +14,10 @@
 // sweep (5 thousand, half of it an FP64 logarithm).  The other teams' passes
 // and M-steps run meanwhile; how many there are is set by shared memory (20 or 28
 // bytes per particle, 16 or 24 with equal weights) and by registers.
-// 16384 3V cells of 572 particles: 284 -> 126 ms against one CTA of 256
+// 16384 3V cells of 572 particles: 285 -> 124 ms against one CTA of 256
 // threads per cell with a fixed tile of 3072 particles (two per SM); 4096 1V
-// cells of 2000: 113 -> 102 ms; 1024 3V cells of 1024 with unequal weights:
-// 41 -> 22 ms.
+// cells of 2000: 113 -> 104 ms; 1024 3V cells of 1024 with unequal weights:
+// 43 -> 24 ms.
 //
 // Component-wise EM (Sec. 2.3, Celeux et al.): the E-step of component k
 // needs the normaliser s_p = sum_j omega_j f_j(v_p) with the *current*

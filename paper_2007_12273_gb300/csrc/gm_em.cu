@@ -8,7 +8,8 @@ namespace gmcr {
 //   * A cell of more than 128 pairs takes 4 warps, up to 5 teams per SM: the
 //     serial M-steps of one cell overlap the passes of the others, and 640
 //     threads leave 96 registers, which the passes need without spilling.
-//     4096 1V cells of 2000 particles, 16384 3V cells of 572 on average (ms):
+//     4096 1V cells of 2000 particles, 16384 3V cells of 572 on average (ms, one
+//     run of the variants on the same inputs):
 //     5 x 128 threads 102, 126; 4 x 128 119, 138; 8 x 64 -, 144; 8 x 128 at
 //     64 registers 109, -; one CTA of 256 threads per cell (two or four per
 //     SM, the same work) 113, 284.
