@@ -101,23 +101,29 @@ __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_
   constexpr int NP = NS <= 4 ? 4 : 16;
   __shared__ double parts[NW][NS][2];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  bool big = false;  // the second turn, for the CTA's big cells
-  int64_t j = (int64_t)blockIdx.x * NW + wid;
+  // the CTA's cells: groups of NW, a warp each, or one where the grid has a CTA per cell
+  const int per = C <= (int64_t)gridDim.x ? 1 : NW;
+  const int64_t step = (int64_t)gridDim.x * per;
+  bool big = false, met = false;  // the second turn, for the CTA's big cells; whether it has any
+  int w = 0;                      // place in the group (second turn)
+  int64_t j = wid < per ? (int64_t)blockIdx.x * per + wid : C;
   for (;;) {
     if (j >= C) {
-      if (big) break;
       // every warp gets here once, and they take the second turn together
-      bool any = false;
-      for (int64_t q = blockIdx.x + threadIdx.x * (int64_t)gridDim.x; q < C; q += NW * 32 * (int64_t)gridDim.x)
-        any = any || cell_off[q + 1] - cell_off[q] > kBigCell;
-      if (!__syncthreads_or(any)) break;
+      if (big || !__syncthreads_or(met)) break;
       big = true;
-      j = blockIdx.x;
-      if (j >= C) break;
+      j = (int64_t)blockIdx.x * per;
     }
     const int64_t jc = j, o = cell_off[jc], end = cell_off[jc + 1];
-    j += (int64_t)gridDim.x * (big ? 1 : NW);
-    if ((end - o > kBigCell) != big) continue;
+    j += step;
+    if (big) {
+      j = ++w == per ? j - per + 1 : jc + 1;
+      w = w == per ? 0 : w;
+    }
+    if ((end - o > kBigCell) != big) {
+      met = true;
+      continue;
+    }
     const int64_t first = big ? o + (int64_t)wid * kSumChunk : o;
     ChunkSum tot;  // sum t on lane t < NS
     for (int64_t c0 = first; c0 < end; c0 += (big ? NW : 1) * kSumChunk) {
@@ -254,9 +260,9 @@ __global__ void __launch_bounds__(NW * 32, D == 3 ? 6 : 8) moments_kernel(int64_
       }
       __syncthreads();
       if (wid == 0 && lane < NS)
-        for (int w = 1; w < NW; ++w) {
-          tot.add(parts[w][lane][0], false);
-          tot.e += parts[w][lane][1];
+        for (int q = 1; q < NW; ++q) {
+          tot.add(parts[q][lane][0], false);
+          tot.e += parts[q][lane][1];
         }
       __syncthreads();
       if (wid != 0) continue;
