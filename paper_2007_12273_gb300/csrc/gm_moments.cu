@@ -89,7 +89,7 @@ __global__ void deposit_combine_kernel(int64_t C, const long long* rec, int orde
 // A cell of more than kBigCell particles is left to a whole CTA, after the
 // others: its chunks go round the CTA's warps, whose sums are added in their
 // order.  With a warp for every cell 152 3V cells of 1e5 particles took 3.66 ms
-// and one of 1e7 338; now 2.13 and 199, 1.8 and 170 of it the deposit.
+// and one of 1e7 338; now 2.15 and 200 (with the deposit, a warp a cell).
 constexpr int kBigCell = 2 * kSumChunk;
 constexpr int kLoads = 4;  // particles a lane whose loads are issued together
 template <int D, int NW, typename VT>
